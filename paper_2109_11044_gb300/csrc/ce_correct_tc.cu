@@ -9,16 +9,15 @@
 //               (f16, bf16 or tf32, each rounded to nearest) and store both in
 //               the 128-byte-swizzled K-major layout the MMA reads;
 //   MMA lane    allocates tensor memory and for every chunk issues tcgen05.mma
-//               (kind::f16 or kind::tf32, FP32 accumulate, M = 128, N = R padded
-//               to 16): A_hi B_hi into the unit's main accumulator, A_hi B_lo and
-//               A_lo B_hi into the tile's cross accumulator, i.e. hi*hi + hi*lo +
-//               lo*hi, the low-precision product plus one refinement pass for its
-//               residual; main accumulators alternate between two buffers, one
-//               unit of at most 512 sites each, and cross accumulators between two
-//               buffers, one tile each;
-//   4 epilogue  tcgen05.ld each finished unit and add it into a running FP32
-//               sum kept in shared memory; after the tile's last unit add
-//               (sum + cross) + last unit, scaled, to y by reductions in L2;
+//               (kind::f16 or kind::tf32, FP32 accumulate, M = 128): A_hi [B_hi | B_lo]
+//               as one product of N = 2 x (R padded to 16) columns, then A_lo B_hi
+//               onto its second half, i.e. hi*hi in the main and hi*lo + lo*hi in the
+//               cross columns, the low-precision product plus one refinement pass
+//               for its residual; accumulators alternate between two buffers, one
+//               unit of at most 512 sites each;
+//   4 epilogue  tcgen05.ld each finished unit and add it (cross, then main columns)
+//               into a running FP32 sum kept in shared memory; after the tile's last
+//               unit add the total, scaled, to y by reductions in L2;
 //   loader lane claims work items (tiles, possibly of several events) and
 //               copies each chunk's pre-split weights sigma^2 B (hi and lo, same
 //               layout) into the stage ring with one bulk async copy.
@@ -26,7 +25,8 @@
 // no producers, the A operand (A^-1 as f16 hi/lo blocks) copied from memory with
 // the B operand, and each work item a K part of a tile written as its own partial.
 // Producers read a chunk's site coordinates (1 KB, shared by every tile)
-// straight from global memory through L1, before they wait for a stage.  A
+// straight from global memory through L1, and evaluate their first rows, before
+// they wait for a stage.  A
 // shared-memory ring refilled by bulk copies would need a proxy fence between
 // the producers' generic reads of a slot and the next async-proxy copy into
 // it; without one, fast refills overwrote slots still being read.
@@ -100,7 +100,7 @@ struct TcArgs {
   uint32_t stage_bytes;        // 32768 (A hi, A lo) + bblock
   uint32_t run_off;            // offset of the epilogue's running sums (128 x Npad floats) after the stages
   uint32_t tmem_cols;          // allocated tensor-memory columns (a power of two >= 4 Npad)
-  uint32_t idesc1;             // instruction descriptor, N = Npad
+  uint32_t idesc1, idesc2;     // instruction descriptors, N = Npad and N = 2 Npad
   float a11, a12, a21, a22;    // anisotropic map of the grid-unit offset (ANISO kernels)
   uint32_t epi_wait;           // bound on the epilogue's waits for an accumulator (try_wait rounds)
   int* status;
@@ -362,7 +362,7 @@ __global__ void __maxnreg__(TcRoles<NPW>::MAXREG) correct_tc_kernel(const __grid
   // first 1024-byte-aligned shared address of the dynamic buffer
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   __shared__ __align__(8) uint64_t full_a[4], full_b[4], empty_bar[4], acc_full[2],
-      acc_empty[2], tile_empty[2], drain_bar, item_full[kItemRing], item_empty[kItemRing];
+      acc_empty[2], drain_bar, item_full[kItemRing], item_empty[kItemRing];
   __shared__ int2 item_slot[kItemRing];
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
@@ -383,8 +383,6 @@ __global__ void __maxnreg__(TcRoles<NPW>::MAXREG) correct_tc_kernel(const __grid
       mbar_init(smem_u32(&item_full[k]), 1);
       mbar_init(smem_u32(&item_empty[k]), kConsumers);
     }
-    mbar_init(smem_u32(&tile_empty[0]), 128);
-    mbar_init(smem_u32(&tile_empty[1]), 128);
     mbar_init(smem_u32(&drain_bar), 1);
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -458,8 +456,13 @@ __global__ void __maxnreg__(TcRoles<NPW>::MAXREG) correct_tc_kernel(const __grid
     // stores overlap the other group's evaluation.
     const int grp = threadIdx.x / Ro::GPROD;
     const int t = threadIdx.x % Ro::GPROD;
-    const int c = t & 7;                  // 16-byte piece of a row: sites SPC c .. SPC c + SPC - 1
-    const int row0 = (t >> 3) * RPT;      // tile rows row0 .. row0+RPT-1
+    // One warp per 16-byte piece of the rows (sites SPC c .. SPC c + SPC - 1), so that a
+    // site record is one address for the warp: with eight pieces and four row groups in a
+    // warp each record load took four passes of the L1 data path instead of one.  Lane:
+    // tile rows base + 8 u, u < RPT; the eight lanes of a store phase hold consecutive
+    // rows, which the swizzle spreads over all banks.
+    const int c = t >> 5;
+    const int base_row = (t & 31) / 8 * 32 + (t & 7);
     // The stage ring advances with every chunk of the block (both groups'), as
     // small counters: no division on the per-chunk path.
     Ring stage_ring(S);
@@ -471,51 +474,42 @@ __global__ void __maxnreg__(TcRoles<NPW>::MAXREG) correct_tc_kernel(const __grid
       if (item.x < 0) break;
       const TcEvent& ev = p.ev[MULTI ? item.x : 0];   // one event: fixed parameter offsets
       const float absb = ev.absb, c1 = ev.c1;
-      // per-row shift of the offset (one node along x per row of the tile); anisotropic:
-      // its image under the map, whose first column is (a11, a21).  Values travel in
-      // pairs of adjacent sites.
-      uint64_t ub[RPT], vb[RPT];
-#pragma unroll
-      for (int u = 0; u < RPT; ++u) {
-        const float x = ANISO ? (float)u * absb * p.a11 : (float)u * absb;
-        const float v = ANISO ? (float)u * absb * p.a21 : 0.f;
-        ub[u] = pack2(x, x);
-        vb[u] = pack2(v, v);
-      }
+      // Offsets are formed from the row's multiple of four, then shifted by the row's
+      // remainder of nodes along x (anisotropic: by the shift's image under the map, whose
+      // first column is (a11, a21)).  Values travel in pairs of adjacent sites.
+      const float rem = (float)(base_row & 3);
+      const float ubf = ANISO ? rem * absb * p.a11 : rem * absb, vbf = ANISO ? rem * absb * p.a21 : 0.f;
+      const uint64_t ub = pack2(ubf, ubf), vb = pack2(vbf, vbf), absb2 = pack2(absb, absb);
       const uint64_t tiny2 = pack2(1e-30f, 1e-30f), scale2 = pack2(kLoScale, kLoScale), c1n = pack2(-c1, -c1);
       // the event's fields in registers (a parameter-space read per use would be slow)
       const int nchunks = ev.nchunks;
-      const float4* __restrict__ sites = reinterpret_cast<const float4*>(ev.sites);
+      const ulonglong2* __restrict__ sites = reinterpret_cast<const ulonglong2*>(ev.sites) + c * SPC;
       const int tpr = ev.tiles_per_row;
       const float fgi = (float)(item.y / tpr);
-      const float fgj0 = (float)((item.y % tpr) * TM + row0);
+      const float fgj0 = (float)((item.y % tpr) * TM + (base_row & ~3));
+      const uint64_t fgi2 = pack2(fgi, fgi);
       for (int kc = 0; kc < nchunks; ++kc, stage_ring.next(), gsel = gsel + 1 == Ro::NGROUP ? 0 : gsel + 1) {
         if (gsel != grp) continue;
-        // isotropic: dx0 = the x offset, dy2 = dy^2; anisotropic: the two components of
-        // the mapped offset (u, v) of the tile's first row
-        uint64_t dx0[SPC / 2], dy2[SPC / 2];
-        const float4* __restrict__ sp = sites + (size_t)kc * TK;
+        // the piece's negated site records, component by component: x integer part and scaled
+        // fraction (nx, nf), then of y; dy: the scaled y offset, isotropic: its square
+        uint64_t nx[SPC / 2], nf[SPC / 2], dy[SPC / 2];
+        const ulonglong2* __restrict__ sp = sites + (size_t)kc * TK;
 #pragma unroll
-        for (int j = 0; j < SPC; j += 2) {
-          float du[2], dv[2];
+        for (int j = 0; j < SPC / 2; j += 2) {
+          const ulonglong2 ox = __ldg(sp + j / 2), of = __ldg(sp + SPC / 4 + j / 2);
+          const ulonglong2 oy = __ldg(sp + SPC / 2 + j / 2), og = __ldg(sp + 3 * (SPC / 4) + j / 2);
+          nx[j] = ox.x;
+          nx[j + 1] = ox.y;
+          nf[j] = of.x;
+          nf[j + 1] = of.y;
+          dy[j] = fma2(add2(fgi2, oy.x), absb2, og.x);
+          dy[j + 1] = fma2(add2(fgi2, oy.y), absb2, og.y);
+        }
+        if (!ANISO) {
 #pragma unroll
-          for (int w = 0; w < 2; ++w) {
-            const float4 o = __ldg(sp + (j + w) * 8 + c);
-            const float dx = fmaf(fgj0 - o.x, absb, -o.y);
-            const float dy = fmaf(fgi - o.z, absb, -o.w);
-            if (ANISO) {
-              du[w] = fmaf(p.a11, dx, p.a12 * dy);
-              dv[w] = fmaf(p.a21, dx, p.a22 * dy);
-            } else {
-              du[w] = dx;
-              dv[w] = fmaf(dy, dy, 1e-30f);
-            }
-          }
-          dx0[j / 2] = pack2(du[0], du[1]);
-          dy2[j / 2] = pack2(dv[0], dv[1]);
+          for (int j = 0; j < SPC / 2; ++j) dy[j] = fma2(dy[j], dy[j], tiny2);
         }
         const int s = stage_ring.slot;
-        if (!mbar_wait(smem_u32(&empty_bar[s]), stage_ring.phase ^ 1u, &abort_flag)) { ok = false; break; }
         const uint32_t st = smem_base + (uint32_t)s * p.stage_bytes;
 #pragma unroll
         for (int h = 0; h < RPT; h += 2) {
@@ -524,13 +518,17 @@ __global__ void __maxnreg__(TcRoles<NPW>::MAXREG) correct_tc_kernel(const __grid
           for (int u = 0; u < 2; ++u)
 #pragma unroll
             for (int j = 0; j < SPC / 2; ++j) {
-              const uint64_t dx = (h + u) ? add2(dx0[j], ub[h + u]) : dx0[j];
+              const float fg = fgj0 + (float)(8 * (h + u));
+              const uint64_t dx = fma2(add2(pack2(fg, fg), nx[j]), absb2, nf[j]);
               uint64_t d2;
               if (ANISO) {
-                const uint64_t dv = (h + u) ? add2(dy2[j], vb[h + u]) : dy2[j];
-                d2 = fma2(dx, dx, fma2(dv, dv, tiny2));
+                const float2 xy0 = unpack2(dx), xy1 = unpack2(dy[j]);
+                const uint64_t du = add2(pack2(fmaf(p.a11, xy0.x, p.a12 * xy1.x), fmaf(p.a11, xy0.y, p.a12 * xy1.y)), ub);
+                const uint64_t dv = add2(pack2(fmaf(p.a21, xy0.x, p.a22 * xy1.x), fmaf(p.a21, xy0.y, p.a22 * xy1.y)), vb);
+                d2 = fma2(du, du, fma2(dv, dv, tiny2));
               } else {
-                d2 = fma2(dx, dx, dy2[j]);
+                const uint64_t du = add2(dx, ub);
+                d2 = fma2(du, du, dy[j]);
               }
               // |b| d (distances are in units of the exponent scale) and 2^-|b| d
               const float2 q = unpack2(d2);
@@ -541,28 +539,36 @@ __global__ void __maxnreg__(TcRoles<NPW>::MAXREG) correct_tc_kernel(const __grid
               // 2^11 C: c1 holds 2^11 a / b, so the factor costs nothing for nu = 3/2
               cv[u][j] = NU3 ? mul2(fma2(c1n, pack2(dd.x, dd.y), scale2), e) : mul2(e, scale2);
             }
+          uint32_t hi[2][4], lo[2][4];
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
-            uint32_t hi[4], lo[4];
             if constexpr (KIND == KIND_TF32) {
 #pragma unroll
               for (int j = 0; j < 2; ++j) {
                 const float2 f = unpack2(cv[u][j]);
-                hi[2 * j] = tf32_round_bits(f.x);
-                hi[2 * j + 1] = tf32_round_bits(f.y);
-                lo[2 * j] = tf32_round_bits(f.x - __uint_as_float(hi[2 * j]));
-                lo[2 * j + 1] = tf32_round_bits(f.y - __uint_as_float(hi[2 * j + 1]));
+                hi[u][2 * j] = tf32_round_bits(f.x);
+                hi[u][2 * j + 1] = tf32_round_bits(f.y);
+                lo[u][2 * j] = tf32_round_bits(f.x - __uint_as_float(hi[u][2 * j]));
+                lo[u][2 * j + 1] = tf32_round_bits(f.y - __uint_as_float(hi[u][2 * j + 1]));
               }
             } else {
 #pragma unroll
-              for (int j = 0; j < 4; ++j) split_pack<F16>(cv[u][j], hi[j], lo[j]);
+              for (int j = 0; j < 4; ++j) split_pack<F16>(cv[u][j], hi[u][j], lo[u][j]);
             }
-            const int row = row0 + h + u;
+          }
+          if (h == 0) {   // the stage is needed only now: the first rows are evaluated before the wait
+            ok = mbar_wait(smem_u32(&empty_bar[s]), stage_ring.phase ^ 1u, &abort_flag);
+            if (!ok) break;
+          }
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const int row = base_row + 8 * (h + u);
             const uint32_t off = st + (uint32_t)row * 128u + ((uint32_t)(c ^ (row & 7)) << 4);
-            sts128(off, hi[0], hi[1], hi[2], hi[3]);
-            sts128(off + 16384u, lo[0], lo[1], lo[2], lo[3]);
+            sts128(off, hi[u][0], hi[u][1], hi[u][2], hi[u][3]);
+            sts128(off + 16384u, lo[u][0], lo[u][1], lo[u][2], lo[u][3]);
           }
         }
+        if (!ok) break;
         fence_proxy_async();
         mbar_arrive(smem_u32(&full_a[s]));
       }
@@ -570,16 +576,14 @@ __global__ void __maxnreg__(TcRoles<NPW>::MAXREG) correct_tc_kernel(const __grid
     if (!ok) raise_abort(&abort_flag, p.status);
   } else if (warp < Ro::MMA) {
     // ------------------------------------------------------------ epilogue
-    // Tensor memory holds two main accumulators (C_hi B_hi) used by alternate units
-    // of ev.drain chunks, each unit summed from zero, and two cross accumulators
-    // (C_hi B_lo + C_lo B_hi, about 2^-11 of the main terms) used by alternate tiles;
-    // the running sum of a tile's finished units is kept in shared memory by this
-    // role (each thread its row: columns in float4 groups, rows adjacent).  No FP32
-    // accumulator in tensor memory therefore runs over more than ev.drain chunks of
-    // the large terms, and the next tile's cross products never wait for this
-    // tile's total.  After the last unit the total is added to y by reductions
-    // performed in L2 (nothing to wait for here; one thread's reductions to one
-    // address apply in program order).
+    // Tensor memory holds two buffers used by alternate units of ev.drain chunks, each
+    // unit summed from zero: Npad main columns (C_hi B_hi) and Npad cross columns
+    // (C_hi B_lo + C_lo B_hi, about 2^-11 of the main terms).  The running sum of a
+    // tile's finished units is kept in shared memory by this role (each thread its row:
+    // columns in float4 groups, rows adjacent), so no FP32 accumulator in tensor memory
+    // runs over more than ev.drain chunks.  After the last unit the total is added to y
+    // by reductions performed in L2 (nothing to wait for here; one thread's reductions
+    // to one address apply in program order).
     const int q = warp & 3;                 // tensor-memory lanes 32q .. 32q+31
     const int row = 32 * q + lane;
     const uint32_t lanes = (uint32_t)(32 * q) << 16;
@@ -625,11 +629,11 @@ __global__ void __maxnreg__(TcRoles<NPW>::MAXREG) correct_tc_kernel(const __grid
           break;
         }
         tc_fence_after();
-        const uint32_t t_main = tmem_base + lanes + (uint32_t)buf * (uint32_t)p.Npad;
-        const uint32_t t_cross = tmem_base + lanes + (2u + (k & 1u)) * (uint32_t)p.Npad;
+        const uint32_t t_main = tmem_base + lanes + (uint32_t)buf * 2u * (uint32_t)p.Npad;
+        const uint32_t t_cross = t_main + (uint32_t)p.Npad;
         const bool first = u == 0, last = u + 1 == units;
         if (last) {
-          // the tile's total: (running sum + cross accumulator) + last unit, scaled
+          // the tile's total: (running sum + cross) + main columns of the last unit, scaled
           float* __restrict__ yp = yg;
           for (int c0 = 0; c0 < p.Npad; c0 += 8) {
             uint32_t r[8], rc[8];
@@ -658,28 +662,26 @@ __global__ void __maxnreg__(TcRoles<NPW>::MAXREG) correct_tc_kernel(const __grid
               }
             }
           }
-          tc_fence_before();
-          mbar_arrive(smem_u32(&tile_empty[k & 1u]));   // this tile's cross accumulator is read
         } else {
-          // running sum (+)= this unit's main accumulator
+          // running sum (+)= this unit's cross, then main columns
           for (int c0 = 0; c0 < p.Npad; c0 += 8) {
-            uint32_t r[8];
+            uint32_t r[8], rc[8];
             tmem_ld8(t_main + (uint32_t)c0, r);
+            tmem_ld8(t_cross + (uint32_t)c0, rc);
             float4 s0 = make_float4(0.f, 0.f, 0.f, 0.f), s1 = s0;
             if (!first) {
               s0 = run4[(c0 >> 2) * TM];
               s1 = run4[((c0 >> 2) + 1) * TM];
             }
             tmem_wait_ld();
-            if (first) {
-              s0 = make_float4(__uint_as_float(r[0]), __uint_as_float(r[1]), __uint_as_float(r[2]), __uint_as_float(r[3]));
-              s1 = make_float4(__uint_as_float(r[4]), __uint_as_float(r[5]), __uint_as_float(r[6]), __uint_as_float(r[7]));
-            } else {
-              s0 = make_float4(s0.x + __uint_as_float(r[0]), s0.y + __uint_as_float(r[1]), s0.z + __uint_as_float(r[2]),
-                               s0.w + __uint_as_float(r[3]));
-              s1 = make_float4(s1.x + __uint_as_float(r[4]), s1.y + __uint_as_float(r[5]), s1.z + __uint_as_float(r[6]),
-                               s1.w + __uint_as_float(r[7]));
+            float sv[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const float cs = first ? __uint_as_float(rc[j]) : sv[j] + __uint_as_float(rc[j]);
+              sv[j] = cs + __uint_as_float(r[j]);
             }
+            s0 = make_float4(sv[0], sv[1], sv[2], sv[3]);
+            s1 = make_float4(sv[4], sv[5], sv[6], sv[7]);
             run4[(c0 >> 2) * TM] = s0;
             run4[((c0 >> 2) + 1) * TM] = s1;
           }
@@ -702,10 +704,6 @@ __global__ void __maxnreg__(TcRoles<NPW>::MAXREG) correct_tc_kernel(const __grid
       if (item.x < 0) break;
       const TcEvent& ev = p.ev[MULTI ? item.x : 0];   // one event: fixed parameter offsets
       if (lane == 0) {
-        // the cross accumulator and the running sum of the previous tile have been read
-        // the cross accumulator of this tile's parity: read by the epilogue two tiles ago
-        if (!mbar_wait(smem_u32(&tile_empty[k & 1u]), ((k >> 1) & 1u) ^ 1u, &abort_flag)) ok = false;
-        const uint32_t t_cross = tmem_base + (2u + (k & 1u)) * (uint32_t)p.Npad;
         uint32_t t_main = tmem_base;
         int kin = 0;   // chunk within the current accumulation unit
         int tile, k0, k1;
@@ -716,7 +714,7 @@ __global__ void __maxnreg__(TcRoles<NPW>::MAXREG) correct_tc_kernel(const __grid
             const int buf = (int)(unit & 1u);
             if (!mbar_wait(smem_u32(&acc_empty[buf]), ((unit >> 1) & 1u) ^ 1u, &abort_flag)) { ok = false; break; }
             tc_fence_after();
-            t_main = tmem_base + (uint32_t)buf * (uint32_t)p.Npad;
+            t_main = tmem_base + (uint32_t)buf * 2u * (uint32_t)p.Npad;
           }
           const int s = ring.slot;
           const uint32_t ph = ring.phase;
@@ -728,16 +726,19 @@ __global__ void __maxnreg__(TcRoles<NPW>::MAXREG) correct_tc_kernel(const __grid
           }
           tc_fence_after();
           const uint32_t base = smem_base + (uint32_t)s * p.stage_bytes;
-          // the unit's main accumulator: C_hi B_hi; the tile's cross accumulator: C_hi B_lo + C_lo B_hi
-          // (all with the covariance tile's factor 2^11)
+          // C_hi [B_hi | B_lo] into the unit's main and cross columns (the two halves of B are
+          // adjacent rows of the stage), C_lo B_hi onto the cross columns (all with the
+          // covariance tile's factor 2^11).  One product of 2 Npad columns reads C_hi from
+          // shared memory once instead of twice: the reads of the operands are the kernel's
+          // largest load on shared memory.
+          const uint32_t t_cross = t_main + (uint32_t)p.Npad;
           const uint64_t da_hi = sw128_desc(base), da_lo = sw128_desc(base + 16384u);
-          const uint64_t db_hi = sw128_desc(base + 32768u), db_lo = sw128_desc(base + 32768u + (uint32_t)p.Npad * 128u);
+          const uint64_t db = sw128_desc(base + 32768u);
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {   // 4 MMAs of 32 bytes of K (16 or 8 sites) per chunk
+          for (int kk = 0; kk < 4; ++kk) {   // 4 steps of 32 bytes of K (16 or 8 sites) per chunk
             const uint64_t o = 2u * kk;   // 32 bytes along K, in the descriptor's 16-byte units
-            mma_issue<KIND>(t_main, da_hi + o, db_hi + o, p.idesc1, (kin > 0 || kk > 0) ? 1u : 0u);
-            mma_issue<KIND>(t_cross, da_hi + o, db_lo + o, p.idesc1, (kc > k0 || kk > 0) ? 1u : 0u);
-            mma_issue<KIND>(t_cross, da_lo + o, db_hi + o, p.idesc1, 1u);
+            mma_issue<KIND>(t_main, da_hi + o, db + o, p.idesc2, (kin > 0 || kk > 0) ? 1u : 0u);
+            mma_issue<KIND>(t_cross, da_lo + o, db + o, p.idesc1, 1u);
           }
           issued = true;
           mma_commit(smem_u32(&empty_bar[s]));
@@ -838,9 +839,9 @@ __global__ void __maxnreg__(TcRoles<NPW>::MAXREG) correct_tc_kernel(const __grid
 // Weights sigma^2 B (rows = realizations, padded to Npad) split into hi + lo of the
 // operand kind (f16 with the power-of-two scale of f16_scale, bf16, or tf32) in the
 // swizzled K-major layout, bblock bytes per chunk of TK sites; and the chunk's site
-// records (x integer part, x fraction * |b|, y integer part, y fraction * |b|), site k
-// of a chunk at slot (k % SPC) * 8 + k / SPC so that the producers' loads do not
-// collide in banks.
+// records, negated: per piece of SPC sites the x integer parts, x fractions * |b|, y
+// integer parts and y fractions * |b|, each SPC floats in a row, so that a 16-byte load
+// gives two pairs of adjacent sites.
 template <int KIND>
 __global__ void prep_b_kernel(const float* __restrict__ B, int ldb, int R, int nobs, int Npad, int nchunks, float scale,
                               const float4* __restrict__ obs, float absb, uint8_t* __restrict__ bout, uint32_t bblock,
@@ -879,7 +880,11 @@ __global__ void prep_b_kernel(const float* __restrict__ B, int ldb, int R, int n
     }
     if (r == 0) {
       const float4 o = obs[q];
-      sout[(size_t)kc * TK + (k % SPC) * 8 + k / SPC] = make_float4(o.x, o.y * absb, o.z, o.w * absb);
+      float* so = reinterpret_cast<float*>(sout + (size_t)kc * TK) + (k / SPC) * 4 * SPC + k % SPC;
+      so[0] = -o.x;
+      so[SPC] = -(o.y * absb);
+      so[2 * SPC] = -o.z;
+      so[3 * SPC] = -(o.w * absb);
     }
   }
 }
@@ -1073,7 +1078,7 @@ int tc_launch(ce_ctx* owner, TcEvent* ev, int nev, int kind, int Npad, bool nu3,
   a.stages = (int)(budget / a.stage_bytes);
   if (a.stages > 4) a.stages = 4;
   if (a.stages < 2) return fail(owner, CE_ERR_ARG, "tensor-core stage does not fit in shared memory");
-  // two main and two cross accumulators: 4 Npad <= 512 columns
+  // two buffers of Npad main and Npad cross columns: 4 Npad <= 512
   uint32_t ncol = 32;
   while (ncol < 4u * (uint32_t)Npad) ncol <<= 1;
   a.tmem_cols = ncol;
@@ -1082,6 +1087,7 @@ int tc_launch(ce_ctx* owner, TcEvent* ev, int nev, int kind, int Npad, bool nu3,
   const uint32_t fmt = (uint32_t)kind;
   const uint32_t ibase = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(TM >> 4) << 24);
   a.idesc1 = ibase | ((uint32_t)(Npad >> 3) << 17);
+  a.idesc2 = ibase | ((uint32_t)(2 * Npad >> 3) << 17);
   a.a11 = (float)ad.a11;
   a.a12 = (float)ad.a12;
   a.a21 = (float)ad.a21;
