@@ -151,10 +151,16 @@ void launch_normals(const uint32_t* ctr, int count, uint64_t seed, float* out, c
 // looked up (once per device) for the current device.
 int static_scratch_resolve();
 
+// ce_inverse.cu
+// In place: the lower triangle of M (np x np, np = n rounded up to 128, identity past n)
+// becomes that of -M^-1 (FP64; CE_ERR_NOT_SPD where a pivot is not positive);
+// *logdet = log det M.  Synchronises s.
+int spd_inverse_f64(ce_ctx* ctx, double* M, int n, cudaStream_t s, double* logdet);
+// The negated, mirrored n x n matrix of that triangle, as an FP32 pair hi + lo of row
+// stride ld, or in place in FP64 when hi is null.
+void launch_finish_inverse(double* M, int n, float* hi, float* lo, int ld, cudaStream_t s);
+
 // ce_linalg.cu
-// FP64 Cholesky of A (n x n, device, destroyed) and A^-1: into ctx->Ainv_hi/lo
-// (and ctx->logdet) when inv_out is null, else returned in FP64 (caller frees).
-int chol_inverse_f64(ce_ctx* ctx, double* A, int n, cudaStream_t s, double** inv_out);
 void gemm64_nn_sub(const double* A, int lda, const double* B, int ldb, double* C, int ldc, int M, int N, int K,
                    cudaStream_t s);
 void launch_solve(ce_ctx* ctx, const float* E, int R, float* B, int ldb, cudaStream_t s);

@@ -220,18 +220,30 @@ __global__ void local_weights_kernel(GridC g, int np, const double* __restrict__
   obs[q] = split_units(sx, sy, g);
 }
 
-// Covariance matrix between two point sets in FP64, plus `diag` on the diagonal
-// when the sets coincide (dst is rows x cols, row-major).
+// Covariance matrix between two point sets in FP64 (dst is rows x cols, row-major).
 __global__ void cov_matrix_kernel(GridC g, const double* __restrict__ a, int rows, const double* __restrict__ b, int cols,
-                                  double diag_add, const double* __restrict__ diag_vec, double* __restrict__ dst) {
+                                  double* __restrict__ dst) {
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (long long)rows * cols) return;
   const int i = (int)(e / cols), j = (int)(e % cols);
   const double dx = a[2 * i] - b[2 * j], dy = a[2 * i + 1] - b[2 * j + 1];
-  double c = matern_d(aniso_dist(dx, dy, g.an), g.sigma2, g.theta, g.nu3);
-  if (diag_vec != nullptr && i == j) c += diag_add + diag_vec[i];
-  else if (i == j && diag_vec == nullptr && diag_add != 0.0) c += diag_add;
-  dst[e] = c;
+  dst[e] = matern_d(aniso_dist(dx, dy, g.an), g.sigma2, g.theta, g.nu3);
+}
+
+// Lower triangle of the prediction matrix of n points in FP64, K + diag(diag_add + diag_vec)
+// (diag_vec may be null), as an np x np array (np >= n) whose rows past n are the identity's.
+// grid.x: rows, grid.y: 256-column pieces.
+__global__ void spd_cov_kernel(GridC g, const double* __restrict__ a, int n, int np, double diag_add,
+                               const double* __restrict__ diag_vec, double* __restrict__ dst) {
+  const int i = blockIdx.x, j = blockIdx.y * blockDim.x + threadIdx.x;
+  if (j > i) return;
+  double c = i == j ? 1.0 : 0.0;
+  if (i < n) {
+    const double dx = a[2 * i] - a[2 * j], dy = a[2 * i + 1] - a[2 * j + 1];
+    c = matern_d(aniso_dist(dx, dy, g.an), g.sigma2, g.theta, g.nu3);
+    if (i == j) c += diag_vec ? diag_add + diag_vec[i] : diag_add;
+  }
+  dst[(long long)i * np + j] = c;
 }
 
 // k nearest nodes of every site (caller order); marks them in `flags`.
@@ -429,6 +441,34 @@ __global__ void permute_rows_kernel(const float* __restrict__ src, float* __rest
   else dst[(long long)r * ld_dst + q] = src[(long long)r * ld_src + perm[q]];
 }
 
+int pad128(int n) { return (n + 127) / 128 * 128; }
+
+void launch_spd_cov(const GridC& g, const double* xy, int n, double diag_add, const double* diag_vec, double* dst,
+                    cudaStream_t s) {
+  const int np = pad128(n);
+  spd_cov_kernel<<<dim3((unsigned)np, (unsigned)((np + 255) / 256)), 256, 0, s>>>(g, xy, n, np, diag_add, diag_vec, dst);
+}
+
+// The inverse of the prediction matrix in A (lower triangle, padded to nobs_pad) as the
+// context's FP32 pair.
+int store_inverse(ce_ctx* ctx, double* A, cudaStream_t s) {
+  const int n = ctx->nobs, ld = ctx->nobs_pad;
+  int st = spd_inverse_f64(ctx, A, n, s, &ctx->logdet);
+  if (st) return st;
+  const size_t bytes = sizeof(float) * (size_t)ld * ld;
+  ctx->Ainv_hi = (float*)dalloc(ctx, bytes);
+  ctx->Ainv_lo = (float*)dalloc(ctx, bytes);
+  if (!ctx->Ainv_hi || !ctx->Ainv_lo) return fail(ctx, CE_ERR_OOM, "inverse");
+  if (n < ld) {
+    CE_CUDA_TRY(cudaMemsetAsync(ctx->Ainv_hi, 0, bytes, s));
+    CE_CUDA_TRY(cudaMemsetAsync(ctx->Ainv_lo, 0, bytes, s));
+  }
+  launch_finish_inverse(A, n, ctx->Ainv_hi, ctx->Ainv_lo, ld, s);
+  CE_CUDA_TRY(cudaGetLastError());
+  CE_CUDA_TRY(cudaStreamSynchronize(s));
+  return CE_OK;
+}
+
 GridC gridc(const ce_ctx* ctx) {
   GridC g;
   g.m = ctx->m;
@@ -523,16 +563,16 @@ int krige_local_setup(ce_ctx* ctx, const double* xy_host, int n, int np, cudaStr
   for (int q = 0; q < n; ++q) { xy_int[2 * q] = xy_host[2 * perm[q]]; xy_int[2 * q + 1] = xy_host[2 * perm[q] + 1]; }
   double* d_xy = (double*)dalloc(ctx, sizeof(double) * 2 * n);
   double* d_kinv = (double*)dalloc(ctx, sizeof(double) * KMAX * KMAX);
-  double* d_A = (double*)dalloc(ctx, sizeof(double) * (size_t)n * n);
+  double* d_A = (double*)dalloc(ctx, sizeof(double) * (size_t)ctx->nobs_pad * ctx->nobs_pad);
   if (!d_xy || !d_kinv || !d_A) { dfree(ctx, d_xy); dfree(ctx, d_kinv); dfree(ctx, d_A); return fail(ctx, CE_ERR_OOM, "local set-up"); }
   CE_CUDA_TRY(cudaMemcpyAsync(ctx->perm, perm.data(), sizeof(int) * n, cudaMemcpyHostToDevice, s));
   CE_CUDA_TRY(cudaMemcpyAsync(d_xy, xy_int.data(), sizeof(double) * 2 * n, cudaMemcpyHostToDevice, s));
   CE_CUDA_TRY(cudaMemsetAsync(ctx->obs, 0, sizeof(float4) * ctx->nobs_pad, s));
   k11_inverse_kernel<<<1, 256, 0, s>>>(g, np, d_kinv);
   local_weights_kernel<<<(n + 127) / 128, 128, 0, s>>>(g, np, d_xy, n, d_kinv, ctx->idx, ctx->W, ctx->phi, ctx->obs, ctx->tau2);
-  cov_matrix_kernel<<<(unsigned)(((long long)n * n + 255) / 256), 256, 0, s>>>(g, d_xy, n, d_xy, n, ctx->tau2, nullptr, d_A);
+  launch_spd_cov(g, d_xy, n, ctx->tau2, nullptr, d_A, s);
   CE_CUDA_TRY(cudaGetLastError());
-  st = chol_inverse_f64(ctx, d_A, n, s, nullptr);
+  st = store_inverse(ctx, d_A, s);
   dfree(ctx, d_kinv);
   dfree(ctx, d_A);
   if (st) { dfree(ctx, d_xy); return st; }
@@ -573,11 +613,11 @@ int krige_nn_setup(ce_ctx* ctx, const double* xy_host, int n, int k, cudaStream_
   ctx->WN = (float*)dalloc(ctx, sizeof(float) * (size_t)nN * n);
   int* d_Jint = (int*)dalloc(ctx, sizeof(int) * nN);
   double* d_nxy = (double*)dalloc(ctx, sizeof(double) * 2 * nN);
-  double* d_A = (double*)dalloc(ctx, sizeof(double) * (size_t)n * n);
+  double* d_A = (double*)dalloc(ctx, sizeof(double) * (size_t)pad128(n) * pad128(n));
   double* d_G = (double*)dalloc(ctx, sizeof(double) * (size_t)nN * n);
   double* d_C = (double*)dalloc(ctx, sizeof(double) * (size_t)nN * n);
   double* d_sig = (double*)dalloc(ctx, sizeof(double) * nN);
-  double* d_AN = (double*)dalloc(ctx, sizeof(double) * (size_t)nN * nN);
+  double* d_AN = (double*)dalloc(ctx, sizeof(double) * (size_t)ctx->nobs_pad * ctx->nobs_pad);
   auto cleanup = [&]() {
     dfree(ctx, d_sites); dfree(ctx, d_Jint); dfree(ctx, d_nxy); dfree(ctx, d_A); dfree(ctx, d_G);
     dfree(ctx, d_C); dfree(ctx, d_sig); dfree(ctx, d_AN);
@@ -589,21 +629,21 @@ int krige_nn_setup(ce_ctx* ctx, const double* xy_host, int n, int k, cudaStream_
   CE_CUDA_TRY(cudaMemsetAsync(ctx->obs, 0, sizeof(float4) * ctx->nobs_pad, s));
   nn_fill_kernel<<<(nN + 127) / 128, 128, 0, s>>>(d_Jint, nN, ctx->m, ctx->x0, ctx->y0, ctx->h, ctx->idx, ctx->W, ctx->obs, d_nxy);
   // A = K_oo + tau^2 I  and its FP64 inverse
-  cov_matrix_kernel<<<(unsigned)(((long long)n * n + 255) / 256), 256, 0, s>>>(g, d_sites, n, d_sites, n, ctx->tau2, nullptr, d_A);
+  launch_spd_cov(g, d_sites, n, ctx->tau2, nullptr, d_A, s);
   CE_CUDA_TRY(cudaGetLastError());
-  double* Ainv = nullptr;
-  if ((st = chol_inverse_f64(ctx, d_A, n, s, &Ainv))) { cleanup(); return st; }
+  double ld_sites = 0.0;
+  if ((st = spd_inverse_f64(ctx, d_A, n, s, &ld_sites))) { cleanup(); return st; }
+  launch_finish_inverse(d_A, n, nullptr, nullptr, 0, s);
   // G = K_No (internal rows), C = -G A^-1, sigma_N^2, WN
-  cov_matrix_kernel<<<(unsigned)(((long long)nN * n + 255) / 256), 256, 0, s>>>(g, d_nxy, nN, d_sites, n, 0.0, nullptr, d_G);
+  cov_matrix_kernel<<<(unsigned)(((long long)nN * n + 255) / 256), 256, 0, s>>>(g, d_nxy, nN, d_sites, n, d_G);
   CE_CUDA_TRY(cudaMemsetAsync(d_C, 0, sizeof(double) * (size_t)nN * n, s));
-  gemm64_nn_sub(d_G, n, Ainv, n, d_C, n, nN, n, n, s);
+  gemm64_nn_sub(d_G, n, d_A, pad128(n), d_C, n, nN, n, n, s);
   nn_finish_kernel<<<(nN + 7) / 8, 256, 0, s>>>(d_C, d_G, nN, n, g.sigma2, ctx->WN, d_sig);
   nn_phi_kernel<<<(nN + 127) / 128, 128, 0, s>>>(d_sig, nN, ctx->tau2, ctx->phi);
   // A_N = K_NN + diag(tau^2 + sigma_N^2)
-  cov_matrix_kernel<<<(unsigned)(((long long)nN * nN + 255) / 256), 256, 0, s>>>(g, d_nxy, nN, d_nxy, nN, ctx->tau2, d_sig, d_AN);
+  launch_spd_cov(g, d_nxy, nN, ctx->tau2, d_sig, d_AN, s);
   CE_CUDA_TRY(cudaGetLastError());
-  dfree(ctx, Ainv);
-  st = chol_inverse_f64(ctx, d_AN, nN, s, nullptr);
+  st = store_inverse(ctx, d_AN, s);
   cleanup();
   if (st) return st;
   ctx->mode = CE_NN;
