@@ -1163,9 +1163,7 @@ int launch_solve_tc(ce_ctx* ctx, const float* E, int R, float* B, int ldb, cudaS
 
 int solve_condsim(ce_ctx* ctx, const float* E, int R, float* B, int ldb, cudaStream_t s, int* launches) {
   if (solve_on_tensor_cores(ctx)) return launch_solve_tc(ctx, E, R, B, ldb, s, launches);
-  launch_solve(ctx, E, R, B, ldb, s);
-  *launches += 2;
-  return CE_OK;
+  return launch_solve(ctx, E, R, B, ldb, s, launches);
 }
 
 }  // namespace ce

@@ -338,7 +338,7 @@ extern "C" int ce_condsim_grad(ce_ctx* ctx, const float* z_dev, int R, uint64_t 
   if (!acc) return fail(ctx, CE_ERR_OOM, "gradient accumulators");
   CE_CUDA_TRY(cudaMemsetAsync(acc, 0, sizeof(double) * 16, s));
   if ((st = fft_unconditional(ctx, R, seed, r_offset, Y, s))) { dfree(ctx, acc); return st; }
-  launch_solve(ctx, ctx->zint, 1, alpha, n, s);   // alpha = A^-1 z
+  if ((st = launch_solve(ctx, ctx->zint, 1, alpha, n, s, nullptr))) { dfree(ctx, acc); return st; }   // alpha = A^-1 z
   const CovF cov = covf(ctx);
   const float inv_sigma = (float)(1.0 / ctx->sigma);
   const long long nW = (long long)(win.i1 - win.i0) * (win.j1 - win.j0);
@@ -354,7 +354,7 @@ extern "C" int ce_condsim_grad(ce_ctx* ctx, const float* z_dev, int R, uint64_t 
                                            c, acc + 0);
   }
   // 2. w = A^-1 c
-  launch_solve(ctx, c, R, w, n, s);
+  if ((st = launch_solve(ctx, c, R, w, n, s, nullptr))) { dfree(ctx, acc); return st; }
   // 3. prediction matrix and log-likelihood
   {
     const size_t shm = sizeof(float) * 2 * (size_t)R * GP_T;

@@ -42,6 +42,8 @@ struct ce_ctx {
   float4* obs = nullptr;    // nobs points in grid units (int part, frac part) x, y; internal order
   float* Ainv_hi = nullptr; // nobs x nobs, internal order
   float* Ainv_lo = nullptr;
+  void* ainv_dig = nullptr; // the pair's 8-bit digit planes (nobs >= kXprodMin)
+  void* xrows = nullptr;    // those of a call's right-hand sides
   double logdet = 0;
   // gradient set-up (local mode), computed on first use
   double* sites64 = nullptr;  // nobs x 2 FP64 site coordinates, internal order
@@ -163,7 +165,20 @@ void launch_finish_inverse(double* M, int n, float* hi, float* lo, int ld, cudaS
 // ce_linalg.cu
 void gemm64_nn_sub(const double* A, int lda, const double* B, int ldb, double* C, int ldc, int M, int N, int K,
                    cudaStream_t s);
-void launch_solve(ce_ctx* ctx, const float* E, int R, float* B, int ldb, cudaStream_t s);
+// B = A^-1 E with the stored pair, through the context's Bpart (and xrows); *launches counts
+// its kernels (may be null).
+int launch_solve(ce_ctx* ctx, const float* E, int R, float* B, int ldb, cudaStream_t s, int* launches);
+// ce_xprod.cu: E A^-1 on the tensor cores from 8-bit digits.  The digit planes of the n x n
+// pair hi + lo (row stride ld), in a buffer of xprod_matrix_bytes(n); those of R rows of E
+// take xprod_rows_bytes(n, R).  launch_xprod writes *kparts <= max_parts partial (sum,
+// compensation) pairs per output to part (kparts x R x n), E's row stride lde.
+size_t xprod_matrix_bytes(int n);
+size_t xprod_rows_bytes(int n, int R);
+void launch_xprod_matrix(const float* hi, const float* lo, int ld, int n, void* buf, cudaStream_t s);
+int launch_xprod(ce_ctx* ctx, const float* E, long long lde, int R, int n, const void* matrix, void* rows, float* part,
+                 int max_parts, int* kparts, cudaStream_t s);
+// From this many rows on the solve takes the tensor-core digits.
+constexpr int kXprodMin = 1800;
 // The context's solve form is the tensor-core one.
 bool solve_on_tensor_cores(const ce_ctx* ctx);
 // B = A^-1 E on the tensor cores (f16 hi/lo operands, FP32 accumulation drained every 512

@@ -464,6 +464,11 @@ int store_inverse(ce_ctx* ctx, double* A, cudaStream_t s) {
     CE_CUDA_TRY(cudaMemsetAsync(ctx->Ainv_lo, 0, bytes, s));
   }
   launch_finish_inverse(A, n, ctx->Ainv_hi, ctx->Ainv_lo, ld, s);
+  if (n >= kXprodMin) {
+    ctx->ainv_dig = dalloc(ctx, xprod_matrix_bytes(n));
+    if (!ctx->ainv_dig) return fail(ctx, CE_ERR_OOM, "digits of the inverse");
+    launch_xprod_matrix(ctx->Ainv_hi, ctx->Ainv_lo, ld, n, ctx->ainv_dig, s);
+  }
   CE_CUDA_TRY(cudaGetLastError());
   CE_CUDA_TRY(cudaStreamSynchronize(s));
   return CE_OK;
@@ -501,6 +506,8 @@ void free_offgrid(ce_ctx* ctx) {
   dfree(ctx, ctx->Ainv_hi); ctx->Ainv_hi = nullptr;
   dfree(ctx, ctx->Ainv_lo); ctx->Ainv_lo = nullptr;
   dfree(ctx, ctx->ainv_blk); ctx->ainv_blk = nullptr;
+  dfree(ctx, ctx->ainv_dig); ctx->ainv_dig = nullptr;
+  dfree(ctx, ctx->xrows); ctx->xrows = nullptr;
   dfree(ctx, ctx->solve_part); ctx->solve_part = nullptr; ctx->solve_part_bytes = 0;
   dfree(ctx, ctx->zint); ctx->zint = nullptr;
   dfree(ctx, ctx->sites64); ctx->sites64 = nullptr;

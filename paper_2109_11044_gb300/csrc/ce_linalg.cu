@@ -231,17 +231,17 @@ __global__ void __launch_bounds__(128) solve_gemm_f32(const float* __restrict__ 
   }
 }
 
-// Bout[r][c] = the KSPLIT partial (sum, compensation) pairs added as an unevaluated
+// Bout[r][c] = the partial (sum, compensation) pairs added as an unevaluated
 // float pair (TwoSum of the sums, the compensations and the TwoSum errors gathered in
 // a second float: FP64 arithmetic is slow on this part), rounded once.
-__global__ void solve_reduce(const float* __restrict__ part, int R, int n, float* __restrict__ Bout, int ldb) {
+__global__ void solve_reduce(const float* __restrict__ part, int parts, int R, int n, float* __restrict__ Bout, int ldb) {
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (long long)R * n) return;
   const long long stride = (long long)R * n;
   const float2* __restrict__ pp = reinterpret_cast<const float2*>(part);
   float hi = 0.f, lo = 0.f;
-#pragma unroll
-  for (int k = 0; k < SV_KSPLIT; ++k) {
+#pragma unroll 4
+  for (int k = 0; k < parts; ++k) {
     const float2 v = pp[k * stride + e];
     const float t = __fadd_rn(hi, v.x);
     const float z = __fsub_rn(t, hi);
@@ -282,17 +282,26 @@ void gemm64_nn_sub(const double* A, int lda, const double* B, int ldb, double* C
   gemm64_sub<<<g, 256, 0, s>>>(A, lda, B, ldb, C, ldc, M, N, K);
 }
 
-void launch_solve(ce_ctx* ctx, const float* E, int R, float* B, int ldb, cudaStream_t s) {
+int launch_solve(ce_ctx* ctx, const float* E, int R, float* B, int ldb, cudaStream_t s, int* launches) {
   const int n = ctx->nobs;
-  dim3 g((n + SV_TC - 1) / SV_TC, (R + SV_TR - 1) / SV_TR, SV_KSPLIT);
-  // the FP32 form keeps pairs (the tightest error); the tensor forms, whose correction
-  // error dominates, sum four hi products per compensated step (a quarter faster)
-  if (ctx->prec == CE_PREC_FP32 || ctx->prec == CE_PREC_FP64)
-    solve_gemm_f32<2><<<g, 128, 0, s>>>(E, R, n, ctx->Ainv_hi, ctx->Ainv_lo, ctx->nobs_pad, ctx->Bpart);
-  else
-    solve_gemm_f32<4><<<g, 128, 0, s>>>(E, R, n, ctx->Ainv_hi, ctx->Ainv_lo, ctx->nobs_pad, ctx->Bpart);
   const long long tot = (long long)R * n;
-  solve_reduce<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(ctx->Bpart, R, n, B, ldb);
+  int parts = SV_KSPLIT;
+  if (ctx->ainv_dig) {
+    const int st = launch_xprod(ctx, E, n, R, n, ctx->ainv_dig, ctx->xrows, ctx->Bpart, SV_KSPLIT, &parts, s);
+    if (st) return st;
+    if (launches) *launches += 1;
+  } else {
+    dim3 g((n + SV_TC - 1) / SV_TC, (R + SV_TR - 1) / SV_TR, SV_KSPLIT);
+    // the FP32 form keeps pairs (the tightest error); the tensor forms, whose correction
+    // error dominates, sum four hi products per compensated step (a quarter faster)
+    if (ctx->prec == CE_PREC_FP32 || ctx->prec == CE_PREC_FP64)
+      solve_gemm_f32<2><<<g, 128, 0, s>>>(E, R, n, ctx->Ainv_hi, ctx->Ainv_lo, ctx->nobs_pad, ctx->Bpart);
+    else
+      solve_gemm_f32<4><<<g, 128, 0, s>>>(E, R, n, ctx->Ainv_hi, ctx->Ainv_lo, ctx->nobs_pad, ctx->Bpart);
+  }
+  solve_reduce<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(ctx->Bpart, parts, R, n, B, ldb);
+  if (launches) *launches += 2;
+  return CE_OK;
 }
 
 void launch_gemm_hilo(const float* E, int R, int n, const float* hi, const float* lo, int lda, float* part, float* out,
@@ -301,7 +310,7 @@ void launch_gemm_hilo(const float* E, int R, int n, const float* hi, const float
   if (compensated) solve_gemm_f32<2><<<g, 128, 0, s>>>(E, R, n, hi, lo, lda, part);
   else solve_gemm_f32<0><<<g, 128, 0, s>>>(E, R, n, hi, lo, lda, part);
   const long long tot = (long long)R * n;
-  solve_reduce<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(part, R, n, out, ldo);
+  solve_reduce<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(part, SV_KSPLIT, R, n, out, ldo);
 }
 
 void launch_gemv_f32(const float* Amat, const float* x, float* y, int rows, int cols, cudaStream_t s) {
