@@ -171,12 +171,12 @@ int launch_solve(ce_ctx* ctx, const float* E, int R, float* B, int ldb, cudaStre
 // ce_xprod.cu: E A^-1 on the tensor cores from 8-bit digits.  The digit planes of the n x n
 // pair hi + lo (row stride ld), in a buffer of xprod_matrix_bytes(n); those of R rows of E
 // take xprod_rows_bytes(n, R).  launch_xprod writes *kparts <= max_parts partial (sum,
-// compensation) pairs per output to part (kparts x R x n), E's row stride lde.
+// compensation) pairs per output to part (kparts x R x n); E's rows of stride lde.
 size_t xprod_matrix_bytes(int n);
 size_t xprod_rows_bytes(int n, int R);
 void launch_xprod_matrix(const float* hi, const float* lo, int ld, int n, void* buf, cudaStream_t s);
-int launch_xprod(ce_ctx* ctx, const float* E, long long lde, int R, int n, const void* matrix, void* rows, float* part,
-                 int max_parts, int* kparts, cudaStream_t s);
+int launch_xprod(ce_ctx* ctx, const float* E, long long lde, int R, int n, const void* matrix, void* rows,
+                 float* part, int max_parts, int* kparts, cudaStream_t s);
 // From this many rows on the solve takes the tensor-core digits.
 constexpr int kXprodMin = 1800;
 // The context's solve form is the tensor-core one.
@@ -187,12 +187,6 @@ int launch_solve_tc(ce_ctx* ctx, const float* E, int R, float* B, int ldb, cudaS
 // The solve of a conditional-simulation call in the form the context selects; returns
 // the status, *launches the kernels it launched.
 int solve_condsim(ce_ctx* ctx, const float* E, int R, float* B, int ldb, cudaStream_t s, int* launches);
-// out (R x n, row stride ldo) = E (R x n) times the symmetric FP32 pair hi + lo (n x n,
-// row stride lda, a multiple of 128), through kSolveKSplit partial products in part
-// (kSolveKSplit x R x n float pairs).  compensated: TwoSum accumulation (the solve
-// that feeds the correction); otherwise per-chunk FP32 sums joined by Kahan compensation.
-void launch_gemm_hilo(const float* E, int R, int n, const float* hi, const float* lo, int lda, float* part, float* out,
-                      int ldo, cudaStream_t s, bool compensated);
 void launch_gemv_f32(const float* Amat, const float* x, float* y, int rows, int cols, cudaStream_t s);
 
 // ce_krige.cu

@@ -81,7 +81,7 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const float* src, bool 
 
 // CHAIN = 2 or 4: the hi products are summed in FP32 CHAIN at a time and each such partial
 // joins the running sum by an error-free TwoSum (the error kept in the compensation with
-// the lo products); CHAIN = 0: plain per-chunk sums joined with Kahan compensation.
+// the lo products).
 template <int CHAIN>
 __global__ void __launch_bounds__(128) solve_gemm_f32(const float* __restrict__ E, int R, int n,
                                                       const float* __restrict__ Ahi, const float* __restrict__ Alo,
@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(128) solve_gemm_f32(const float* __restrict__ 
             comp[i][j] = fmaf(eb[i], lb[j], fmaf(ea[i], la[j], comp[i][j] + es));
           }
       }
-    } else if constexpr (CHAIN == 4) {
+    } else {
 #pragma unroll 1
       for (int kk = 0; kk < SV_KC; kk += 4) {   // SV_KC is a multiple of 4; rows past kend were copied as zeros
         float hv[4][4], lv[4][4];
@@ -184,37 +184,6 @@ __global__ void __launch_bounds__(128) solve_gemm_f32(const float* __restrict__ 
           }
         }
       }
-    } else {
-      // plain form: per chunk the hi and lo products accumulate in FP32 (apart, so the lo
-      // part is not absorbed); chunk sums join the running sum with Kahan compensation
-      float ph[4][4], pl[4][4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) { ph[i][j] = 0.f; pl[i][j] = 0.f; }
-#pragma unroll 8
-      for (int kk = 0; kk < SV_KC; ++kk) {
-        const float4 h4 = *reinterpret_cast<const float4*>(&Hs[bf][kk][tx * 4]);
-        const float4 l4 = *reinterpret_cast<const float4*>(&Ls[bf][kk][tx * 4]);
-        const float ev[4] = {Es[bf][ty * 4][kk], Es[bf][ty * 4 + 1][kk], Es[bf][ty * 4 + 2][kk], Es[bf][ty * 4 + 3][kk]};
-        const float hv[4] = {h4.x, h4.y, h4.z, h4.w}, lv[4] = {l4.x, l4.y, l4.z, l4.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            ph[i][j] = fmaf(ev[i], hv[j], ph[i][j]);
-            pl[i][j] = fmaf(ev[i], lv[j], pl[i][j]);
-          }
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {   // Kahan: sum += (hi part + lo part); comp holds the negated error
-          const float yv = (ph[i][j] + pl[i][j]) + comp[i][j];
-          const float t = sum[i][j] + yv;
-          comp[i][j] = yv - (t - sum[i][j]);
-          sum[i][j] = t;
-        }
     }
     __syncthreads();
   }
@@ -302,15 +271,6 @@ int launch_solve(ce_ctx* ctx, const float* E, int R, float* B, int ldb, cudaStre
   solve_reduce<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(ctx->Bpart, parts, R, n, B, ldb);
   if (launches) *launches += 2;
   return CE_OK;
-}
-
-void launch_gemm_hilo(const float* E, int R, int n, const float* hi, const float* lo, int lda, float* part, float* out,
-                      int ldo, cudaStream_t s, bool compensated) {
-  dim3 g((n + SV_TC - 1) / SV_TC, (R + SV_TR - 1) / SV_TR, SV_KSPLIT);
-  if (compensated) solve_gemm_f32<2><<<g, 128, 0, s>>>(E, R, n, hi, lo, lda, part);
-  else solve_gemm_f32<0><<<g, 128, 0, s>>>(E, R, n, hi, lo, lda, part);
-  const long long tot = (long long)R * n;
-  solve_reduce<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(part, SV_KSPLIT, R, n, out, ldo);
 }
 
 void launch_gemv_f32(const float* Amat, const float* x, float* y, int rows, int cols, cudaStream_t s) {

@@ -353,7 +353,9 @@ __global__ void __launch_bounds__(kThreads) xprod_kernel(const __grid_constant__
         for (int j = 0; j < 64; ++j) {
           if (j < ncol && rb + j < p.R) {
             const float sc = p.bscale[rb + j];
-            dst[(size_t)(rb + j) * p.n] = make_float2(hi[j] * as * sc, lo[j] * as * sc);
+            float h = hi[j];   // a normalised pair: the low part is below half an ulp of the value
+            const float l = two_sum(h, lo[j]);
+            dst[(size_t)(rb + j) * p.n] = make_float2(h * as * sc, l * as * sc);
           }
         }
       }
@@ -394,8 +396,8 @@ size_t xprod_rows_bytes(int n, int R) {
   return (size_t)nb * nchunks_of(n) * kBPlanes * np * 128u + sizeof(float) * (size_t)nb * np;
 }
 
-int launch_xprod(ce_ctx* ctx, const float* E, long long lde, int R, int n, const void* matrix, void* rows, float* part,
-                 int max_parts, int* kparts_out, cudaStream_t s) {
+int launch_xprod(ce_ctx* ctx, const float* E, long long lde, int R, int n, const void* matrix, void* rows,
+                 float* part, int max_parts, int* kparts_out, cudaStream_t s) {
   const int np = block_rows(R), nb = (R + np - 1) / np, nc = nchunks_of(n), mt = mtiles_of(n);
   XArgs a;
   a.a = static_cast<const uint8_t*>(matrix);
