@@ -16,6 +16,7 @@
 // and the last term is evaluated per realization pair in Fourier space:
 // <h_{2p}, d Re w> + <h_{2p+1}, d Im w> = sum_a ds_a Re(eps_a Y_a) with
 // Y = DFT2(h_{2p} - i h_{2p+1}) and s = sqrt(lambda / N).
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -67,56 +68,105 @@ struct Window {
   int i0, i1, j0, j1;
 };
 
-// c[r][q] = f sum_{g in W} C(g, s_q) v_r(g) and, into acc[0..1], the correction
-// term f sum_{g, q} (2 C / sigma, dC / dtheta)(g, q) sum_r v_r(g) B_r(q).
-// Block: 32 sites (internal order) x a slice of the window nodes; 256 threads.
-constexpr int GW_Q = 32, GW_G = 64;
+// Adjoint of the correction over the window: csum[r][q] = sum_{g in W} C(g, s_q) v_r(g) and
+// dsum[r][q] = sum_{g in W} dC/dtheta(g, s_q) v_r(g) (FP64 sums of the blocks' FP32 parts).
+// The correction's own parameter terms are then sums over r, q alone:
+// sum_{g,q} (2 C / sigma, dC / dtheta)(g, q) sum_r v_r(g) B_r(q) = sum_{r,q} B_r(q) (2 csum / sigma, dsum).
+//
+// Block: QT sites (internal order) x RT realizations x a slice of the window's nodes, 256
+// threads of 4 sites x 8 realizations (packed pairs).  Per chunk of GK nodes the two
+// covariance tiles and the fields' values are put in shared memory; the products of two
+// chunks (64 nodes) accumulate in FP32 and join a Kahan sum.  FP32-bound: 1.5e10
+// multiply-adds at 40000 nodes, 3000 sites, R = 64.  (Before, each of the 256 threads read
+// every operand of a multiply-add from shared memory, and the parameter terms were a second
+// contraction over (g, q, r): 7.1 ms there.)
+constexpr int GK = 32;
 
-__global__ void __launch_bounds__(256) grad_window_kernel(const float* __restrict__ v, int m, Window win, int R,
-                                                          const float4* __restrict__ obs, int nobs,
-                                                          const float* __restrict__ B, int ldb, CovF cov, float f,
-                                                          float inv_sigma, float* __restrict__ c, double* __restrict__ acc) {
-  extern __shared__ float gsm[];
-  float* Bs = gsm;                        // [R][GW_Q]
-  float* Vs = Bs + R * GW_Q;              // [R][GW_G]
-  float* Cs = Vs + R * GW_G;              // [GW_Q][GW_G]
-  float* Ds = Cs + GW_Q * GW_G;           // [GW_Q][GW_G]
-  __shared__ double red[32];
-  const int q0 = blockIdx.x * GW_Q;
+__device__ __forceinline__ uint64_t dup2(float x) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(x));
+  return d;
+}
+__device__ __forceinline__ float2 halves(uint64_t v) {
+  float2 d;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(v));
+  return d;
+}
+__device__ __forceinline__ void fma2_into(uint64_t& acc, uint64_t a, uint64_t b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+
+template <int RT>
+struct GradTile {
+  static constexpr int TR = RT / 8;         // threads along the realizations
+  static constexpr int QT = 256 / TR * 4;   // sites per block
+  static constexpr int LV = RT + 4;         // row stride of the fields' values (16-byte aligned)
+  static constexpr size_t smem = sizeof(float) * (size_t)GK * (2 * QT + LV);
+};
+
+template <int RT>
+__global__ void __launch_bounds__(256, 1) grad_window_kernel(const float* __restrict__ v, int m, Window win, int R,
+                                                             const float4* __restrict__ obs, int nobs, CovF cov,
+                                                             double* __restrict__ csum, double* __restrict__ dsum) {
+  using T = GradTile<RT>;
+  constexpr int QT = T::QT, LV = T::LV;
+  extern __shared__ __align__(16) float gsm[];
+  float* Cs = gsm;                 // [GK][QT]
+  float* Ds = Cs + GK * QT;        // [GK][QT]
+  float* Vs = Ds + GK * QT;        // [GK][LV]
+  const int q0 = blockIdx.x * QT;
   const int wj = win.j1 - win.j0;
   const long long nW = (long long)(win.i1 - win.i0) * wj;
   const long long per = (nW + gridDim.y - 1) / gridDim.y;
   const long long g_beg = blockIdx.y * per, g_end = min(nW, g_beg + per);
   const long long M = (long long)m * m;
-  for (int e = threadIdx.x; e < R * GW_Q; e += blockDim.x) {
-    const int r = e / GW_Q, qq = e % GW_Q;
-    Bs[e] = (q0 + qq < nobs) ? B[(long long)r * ldb + q0 + qq] : 0.f;
-  }
-  const int tq = threadIdx.x % GW_Q, tr = threadIdx.x / GW_Q;   // 8 realization groups
-  constexpr int RMAX = 16;                                        // R <= 128
-  float cacc[RMAX];
+  const int tr = threadIdx.x % T::TR, tq = threadIdx.x / T::TR;
+  uint64_t pc[4][4], pd[4][4];     // products of the current chunks: site x pair of realizations
+  float sc[4][8], sd[4][8], ec[4][8], ed[4][8];   // Kahan sums
 #pragma unroll
-  for (int k = 0; k < RMAX; ++k) cacc[k] = 0.f;
-  double ks = 0.0, kt = 0.0;
-  for (long long gb = g_beg; gb < g_end; gb += GW_G) {
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) sc[i][j] = sd[i][j] = ec[i][j] = ed[i][j] = 0.f;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) pc[i][j] = pd[i][j] = 0;
+  auto kahan = [](float& s, float& e, float x) {
+    const float y = __fsub_rn(x, e), t = __fadd_rn(s, y);
+    e = __fsub_rn(__fsub_rn(t, s), y);
+    s = t;
+  };
+  auto join = [&]() {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float2 c = halves(pc[i][j]), d = halves(pd[i][j]);
+        kahan(sc[i][2 * j], ec[i][2 * j], c.x);
+        kahan(sc[i][2 * j + 1], ec[i][2 * j + 1], c.y);
+        kahan(sd[i][2 * j], ed[i][2 * j], d.x);
+        kahan(sd[i][2 * j + 1], ed[i][2 * j + 1], d.y);
+        pc[i][j] = pd[i][j] = 0;
+      }
+  };
+  int odd = 0;
+  for (long long gb = g_beg; gb < g_end; gb += GK, odd ^= 1) {
     __syncthreads();
-    for (int e = threadIdx.x; e < R * GW_G; e += blockDim.x) {
-      const int r = e / GW_G, gg = e % GW_G;
+    for (int e = threadIdx.x; e < GK * RT; e += 256) {
+      const int gg = e % GK, r = e / GK;
       const long long gw = gb + gg;
       float val = 0.f;
-      if (gw < g_end) {
-        const int gi = win.i0 + (int)(gw / wj), gj = win.j0 + (int)(gw % wj);
-        val = v[(long long)r * M + (long long)gi * m + gj];
-      }
-      Vs[e] = val;
+      if (gw < g_end && r < R)
+        val = v[(long long)r * M + (long long)(win.i0 + (int)(gw / wj)) * m + win.j0 + (int)(gw % wj)];
+      Vs[gg * LV + r] = val;
     }
-    for (int e = threadIdx.x; e < GW_Q * GW_G; e += blockDim.x) {
-      const int qq = e / GW_G, gg = e % GW_G;
+    for (int e = threadIdx.x; e < GK * QT; e += 256) {
+      const int gg = e / QT, qq = e % QT;
       const long long gw = gb + gg;
       float cv = 0.f, dv = 0.f;
       if (gw < g_end && q0 + qq < nobs) {
         const int gi = win.i0 + (int)(gw / wj), gj = win.j0 + (int)(gw % wj);
-        const float4 s = obs[q0 + qq];
+        const float4 s = __ldg(obs + q0 + qq);
         const float dx = ((float)gj - s.x) - s.y, dy = ((float)gi - s.z) - s.w;
         cov_and_dtheta(sqrtf(dx * dx + dy * dy), cov, cv, dv);
       }
@@ -124,35 +174,72 @@ __global__ void __launch_bounds__(256) grad_window_kernel(const float* __restric
       Ds[e] = dv;
     }
     __syncthreads();
-    // adjoint of the correction, thread (tq, tr): realizations tr, tr + 8, ...
-    for (int gg = 0; gg < GW_G; ++gg) {
-      const float cv = Cs[tq * GW_G + gg];
+#pragma unroll 2
+    for (int gg = 0; gg < GK; ++gg) {
+      const float4 c4 = *reinterpret_cast<const float4*>(Cs + gg * QT + tq * 4);
+      const float4 d4 = *reinterpret_cast<const float4*>(Ds + gg * QT + tq * 4);
+      const ulonglong2 va = *reinterpret_cast<const ulonglong2*>(Vs + gg * LV + tr * 8);
+      const ulonglong2 vb = *reinterpret_cast<const ulonglong2*>(Vs + gg * LV + tr * 8 + 4);
+      const float c[4] = {c4.x, c4.y, c4.z, c4.w}, d[4] = {d4.x, d4.y, d4.z, d4.w};
+      const uint64_t vv[4] = {va.x, va.y, vb.x, vb.y};
 #pragma unroll
-      for (int k = 0; k < RMAX; ++k) {
-        const int r = tr + 8 * k;
-        if (r < R) cacc[k] = fmaf(cv, Vs[r * GW_G + gg], cacc[k]);
+      for (int i = 0; i < 4; ++i) {
+        const uint64_t c2 = dup2(c[i]), d2 = dup2(d[i]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          fma2_into(pc[i][j], c2, vv[j]);
+          fma2_into(pd[i][j], d2, vv[j]);
+        }
       }
     }
-    // correction term: 8 (g, q) pairs per thread
-    for (int e = threadIdx.x; e < GW_Q * GW_G; e += blockDim.x) {
-      const int qq = e / GW_G, gg = e % GW_G;
-      float gsum = 0.f;
-      for (int r = 0; r < R; ++r) gsum = fmaf(Vs[r * GW_G + gg], Bs[r * GW_Q + qq], gsum);
-      ks += (double)(2.0f * inv_sigma * Cs[e]) * gsum;
-      kt += (double)Ds[e] * gsum;
+    if (odd) join();
+  }
+  join();
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int q = q0 + tq * 4 + i;
+    if (q >= nobs) continue;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int r = tr * 8 + j;
+      if (r >= R) continue;
+      atomicAdd(csum + (long long)r * nobs + q, (double)sc[i][j] - (double)ec[i][j]);
+      atomicAdd(dsum + (long long)r * nobs + q, (double)sd[i][j] - (double)ed[i][j]);
     }
   }
-  if (q0 + tq < nobs) {
-#pragma unroll
-    for (int k = 0; k < RMAX; ++k) {
-      const int r = tr + 8 * k;
-      if (r < R) atomicAdd(c + (long long)r * nobs + q0 + tq, f * cacc[k]);
-    }
+}
+
+// c = f csum (FP32, the right-hand sides of w = A^-1 c) and acc[0..1] += f sum_{r,q} B_r(q)
+// (2 csum / sigma, dsum).
+__global__ void __launch_bounds__(256) grad_window_join_kernel(const double* __restrict__ csum, const double* __restrict__ dsum,
+                                                               const float* __restrict__ B, int ldb, int R, int nobs, float f,
+                                                               float inv_sigma, float* __restrict__ c, double* __restrict__ acc) {
+  __shared__ double red[32];
+  double ks = 0.0, kt = 0.0;
+  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < (long long)R * nobs;
+       e += (long long)gridDim.x * blockDim.x) {
+    const int r = (int)(e / nobs), q = (int)(e % nobs);
+    const double b = (double)B[(long long)r * ldb + q];
+    ks += b * csum[e];
+    kt += b * dsum[e];
+    c[e] = (float)((double)f * csum[e]);
   }
   const double a0 = block_sum(ks, red);
-  if (threadIdx.x == 0) atomicAdd(acc + 0, (double)f * a0);
+  if (threadIdx.x == 0) atomicAdd(acc + 0, (double)f * 2.0 * (double)inv_sigma * a0);
   const double a1 = block_sum(kt, red);
   if (threadIdx.x == 0) atomicAdd(acc + 1, (double)f * a1);
+}
+
+template <int RT>
+int launch_grad_window(const float* v, int m, Window win, int R, const float4* obs, int nobs, CovF cov, double* csum,
+                       double* dsum, long long nW, int nsm, cudaStream_t s) {
+  using T = GradTile<RT>;
+  CE_CUDA_TRY(cudaFuncSetAttribute(grad_window_kernel<RT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem));
+  const int qb = (nobs + T::QT - 1) / T::QT;
+  // slices of the window: two blocks per SM in turn, at least 64 nodes each
+  const int splits = (int)std::max<long long>(1, std::min<long long>(2 * nsm / qb, nW / 64));
+  grad_window_kernel<RT><<<dim3((unsigned)qb, (unsigned)splits), 256, T::smem, s>>>(v, m, win, R, obs, nobs, cov, csum, dsum);
+  return CE_OK;
 }
 
 // sum over sites i, j of dA_ij (a_i a_j / 2 - Ainv_ij / 2 - sum_r w_r,i B_r,j), for
@@ -322,14 +409,17 @@ extern "C" int ce_condsim_grad(ce_ctx* ctx, const float* z_dev, int R, uint64_t 
   if ((st = ce_condsim(ctx, z_dev, R, seed, r_offset, out_dev, stream))) return st;
   const int n = ctx->nobs;
   const long long M = (long long)ctx->m * ctx->m;
-  const size_t need = sizeof(float) * ((size_t)R * M * 2 + (size_t)R * n * 2 + (size_t)n + 8);
+  // the FP64 sums first, so that they are aligned
+  const size_t need = sizeof(double) * (size_t)R * n * 2 + sizeof(float) * ((size_t)R * M * 2 + (size_t)R * n * 2 + (size_t)n + 8);
   if (ctx->grad_bytes < need) {
     dfree(ctx, ctx->grad_buf);
     ctx->grad_buf = (float*)dalloc(ctx, need);
     ctx->grad_bytes = ctx->grad_buf ? need : 0;
     if (!ctx->grad_buf) return fail(ctx, CE_ERR_OOM, "gradient buffers");
   }
-  float* Y = ctx->grad_buf;                 // R x M: the unconditional fields again
+  double* csum = reinterpret_cast<double*>(ctx->grad_buf);   // R x n each
+  double* dsum = csum + (size_t)R * n;
+  float* Y = reinterpret_cast<float*>(dsum + (size_t)R * n);   // R x M: the unconditional fields again
   float* H = Y + (size_t)R * M;             // R x M: h_r
   float* c = H + (size_t)R * M;             // R x n
   float* w = c + (size_t)R * n;             // R x n
@@ -344,14 +434,16 @@ extern "C" int ce_condsim_grad(ce_ctx* ctx, const float* z_dev, int R, uint64_t 
   const long long nW = (long long)(win.i1 - win.i0) * (win.j1 - win.j0);
   const float f = (float)(2.0 / ((double)R * (double)nW));
   // 1. adjoint of the correction over the window
-  CE_CUDA_TRY(cudaMemsetAsync(c, 0, sizeof(float) * (size_t)R * n, s));
+  CE_CUDA_TRY(cudaMemsetAsync(csum, 0, sizeof(double) * (size_t)R * n * 2, s));
   {
-    const size_t shm = sizeof(float) * ((size_t)R * GW_Q + (size_t)R * GW_G + 2 * GW_Q * GW_G);
-    CE_CUDA_TRY(cudaFuncSetAttribute(grad_window_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-    int splits = (int)std::max<long long>(1, std::min<long long>(64, nW / 2048));
-    dim3 g((n + GW_Q - 1) / GW_Q, splits);
-    grad_window_kernel<<<g, 256, shm, s>>>(out_dev, ctx->m, win, R, ctx->obs, n, ctx->Bm, ctx->nobs_pad, cov, f, inv_sigma,
-                                           c, acc + 0);
+    int nsm = 0, dev = 0;
+    CE_CUDA_TRY(cudaGetDevice(&dev));
+    CE_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    auto launch = R <= 16 ? launch_grad_window<16>
+                          : (R <= 32 ? launch_grad_window<32> : (R <= 64 ? launch_grad_window<64> : launch_grad_window<128>));
+    if ((st = launch(out_dev, ctx->m, win, R, ctx->obs, n, cov, csum, dsum, nW, nsm, s))) { dfree(ctx, acc); return st; }
+    grad_window_join_kernel<<<std::min(nsm * 2, (int)(((long long)R * n + 255) / 256)), 256, 0, s>>>(
+        csum, dsum, ctx->Bm, ctx->nobs_pad, R, n, f, inv_sigma, c, acc + 0);
   }
   // 2. w = A^-1 c
   if ((st = launch_solve(ctx, c, R, w, n, s, nullptr))) { dfree(ctx, acc); return st; }
