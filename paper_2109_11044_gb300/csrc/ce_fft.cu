@@ -542,7 +542,15 @@ adj_rows_kernel(const float2* __restrict__ T, int m, const float2* __restrict__ 
   }
   __syncthreads();
   fft_lines_smem<P, ROWS, kNT>(sm, tw);
-  double st = 0.0, ss = 0.0;
+  // Sums as FP32 pairs with error-free transformations (two FP64 multiply-adds and their
+  // conversions per element were the kernel's bound on this part).
+  float2 pt = make_float2(0.f, 0.f), ps = make_float2(0.f, 0.f);
+  auto add_product = [](float2& acc, float x, float y) {
+    const float p = __fmul_rn(x, y), pe = fmaf(x, y, -p);
+    const float t = __fadd_rn(acc.x, p), z = __fsub_rn(t, acc.x);
+    acc.y += __fadd_rn(__fsub_rn(acc.x, __fsub_rn(t, z)), __fsub_rn(p, z)) + pe;
+    acc.x = t;
+  };
   for (int e = threadIdx.x; e < ROWS * P; e += kNT) {
     const int row = e / P, b = e % P;
     const int a = a0 + row;
@@ -552,9 +560,10 @@ adj_rows_kernel(const float2* __restrict__ T, int m, const float2* __restrict__ 
     const float2 y = sm[e];
     const float re = z.x * y.x - z.y * y.y;
     const long long o = (long long)a * P + b;
-    st += (double)dsdt[o] * re;
-    ss += (double)(sqrt_lam[o] * inv_sigma) * re;
+    add_product(pt, dsdt[o], re);
+    add_product(ps, sqrt_lam[o] * inv_sigma, re);
   }
+  double st = (double)pt.x + (double)pt.y, ss = (double)ps.x + (double)ps.y;
   for (int o = 16; o; o >>= 1) {
     st += __shfl_xor_sync(0xffffffffu, st, o);
     ss += __shfl_xor_sync(0xffffffffu, ss, o);

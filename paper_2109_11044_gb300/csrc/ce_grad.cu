@@ -114,6 +114,7 @@ __global__ void __launch_bounds__(256, 1) grad_window_kernel(const float* __rest
   float* Cs = gsm;                 // [GK][QT]
   float* Ds = Cs + GK * QT;        // [GK][QT]
   float* Vs = Ds + GK * QT;        // [GK][LV]
+  __shared__ int2 node[GK];        // grid row and column of the chunk's nodes, (-1, -1) past the slice
   const int q0 = blockIdx.x * QT;
   const int wj = win.j1 - win.j0;
   const long long nW = (long long)(win.i1 - win.i0) * wj;
@@ -152,26 +153,31 @@ __global__ void __launch_bounds__(256, 1) grad_window_kernel(const float* __rest
   int odd = 0;
   for (long long gb = g_beg; gb < g_end; gb += GK, odd ^= 1) {
     __syncthreads();
+    if (threadIdx.x < GK) {   // one division per node, not one per element
+      const long long gw = gb + threadIdx.x;
+      const int gi = (int)(gw / wj), gj = (int)(gw % wj);
+      node[threadIdx.x] = gw < g_end ? make_int2(win.i0 + gi, win.j0 + gj) : make_int2(-1, -1);
+    }
+    __syncthreads();
     for (int e = threadIdx.x; e < GK * RT; e += 256) {
       const int gg = e % GK, r = e / GK;
-      const long long gw = gb + gg;
-      float val = 0.f;
-      if (gw < g_end && r < R)
-        val = v[(long long)r * M + (long long)(win.i0 + (int)(gw / wj)) * m + win.j0 + (int)(gw % wj)];
-      Vs[gg * LV + r] = val;
+      const int2 g = node[gg];
+      Vs[gg * LV + r] = g.x >= 0 && r < R ? v[(long long)r * M + (long long)g.x * m + g.y] : 0.f;
     }
-    for (int e = threadIdx.x; e < GK * QT; e += 256) {
-      const int gg = e / QT, qq = e % QT;
-      const long long gw = gb + gg;
-      float cv = 0.f, dv = 0.f;
-      if (gw < g_end && q0 + qq < nobs) {
-        const int gi = win.i0 + (int)(gw / wj), gj = win.j0 + (int)(gw % wj);
-        const float4 s = __ldg(obs + q0 + qq);
-        const float dx = ((float)gj - s.x) - s.y, dy = ((float)gi - s.z) - s.w;
-        cov_and_dtheta(sqrtf(dx * dx + dy * dy), cov, cv, dv);
+    for (int qq = threadIdx.x % QT; qq < QT; qq += 256) {
+      const bool live = q0 + qq < nobs;
+      const float4 s = __ldg(obs + (live ? q0 + qq : 0));
+      // (QT < 256: the threads past QT take other nodes of the same sites)
+      for (int gg = QT < 256 ? threadIdx.x / QT : 0; gg < GK; gg += QT < 256 ? 256 / QT : 1) {
+        const int2 g = node[gg];
+        float cv = 0.f, dv = 0.f;
+        if (live && g.x >= 0) {
+          const float dx = ((float)g.y - s.x) - s.y, dy = ((float)g.x - s.z) - s.w;
+          cov_and_dtheta(sqrtf(dx * dx + dy * dy), cov, cv, dv);
+        }
+        Cs[gg * QT + qq] = cv;
+        Ds[gg * QT + qq] = dv;
       }
-      Cs[e] = cv;
-      Ds[e] = dv;
     }
     __syncthreads();
 #pragma unroll 2
