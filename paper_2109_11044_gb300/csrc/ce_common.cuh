@@ -68,6 +68,33 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, const PhiloxKeys& K) {
   return c;
 }
 
+// Two FP32 results per instruction; each half is rounded as the scalar instruction rounds it.
+__device__ __forceinline__ float2 fma_f2(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmov.b64 z, {%6, %7};\n\tfma.rn.f32x2 x, x, y, z;\n\tmov.b64 {%0, %1}, x;\n\t}"
+      : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
+__device__ __forceinline__ float2 mul_f2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmul.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+      : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+__device__ __forceinline__ float2 both2(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float2 add_f2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tadd.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+      : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+__device__ __forceinline__ float2 sub_f2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tsub.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+      : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+
 // Two uint32 words -> two N(0,1) values by Box-Muller, with u = (x + 1/2) 2^-32.
 // ln(u) for u < 1/2 comes from the fast log (3 ulp there); for u >= 1/2 it is
 // ln(1 - q) with q = (~x + 1/2) 2^-32 formed without cancellation: the fast log
@@ -78,8 +105,8 @@ __device__ __forceinline__ float2 box_muller(uint32_t a, uint32_t b) {
   // Branch-free (the three cases select, so a warp never runs two of them):
   // the fast log of u or of 1 - q, and the series for u close to 1.
   const bool upper = a >= 0x80000000u;
-  const float q = fmaf((float)(~a), 0x1p-32f, 0x1p-33f);
-  const float larg = upper ? 1.0f - q : fmaf((float)a, 0x1p-32f, 0x1p-33f);
+  const float q = fmaf((float)min(a, ~a), 0x1p-32f, 0x1p-33f);   // of a itself in the lower half
+  const float larg = upper ? 1.0f - q : q;
   const float lfast = __logf(larg);
   float p = fmaf(q, 1.0f / 7.0f, 1.0f / 6.0f);
   p = fmaf(q, p, 0.2f);
@@ -96,6 +123,32 @@ __device__ __forceinline__ float2 box_muller(uint32_t a, uint32_t b) {
   float s, c;
   __sincosf(th, &s, &c);
   return make_float2(-rad * c, -rad * s);
+}
+
+// Both pairs of one counter's four words, scaled: z0 = s0 box_muller(x.x, x.y) and
+// z1 = s1 box_muller(x.z, x.w), to the bit, with the series and the angles two at a time.
+__device__ __forceinline__ void box_muller2(uint4 x, float s0, float s1, float2& z0, float2& z1) {
+  const bool u0 = x.x >= 0x80000000u, u1 = x.z >= 0x80000000u;
+  const float2 q = fma_f2(make_float2((float)min(x.x, ~x.x), (float)min(x.z, ~x.z)), both2(0x1p-32f), both2(0x1p-33f));
+  const float l0 = __logf(u0 ? 1.0f - q.x : q.x), l1 = __logf(u1 ? 1.0f - q.y : q.y);
+  float2 p = fma_f2(q, both2(1.0f / 7.0f), both2(1.0f / 6.0f));
+  p = fma_f2(q, p, both2(0.2f));
+  p = fma_f2(q, p, both2(0.25f));
+  p = fma_f2(q, p, both2(1.0f / 3.0f));
+  p = fma_f2(q, p, both2(0.5f));
+  p = fma_f2(q, p, both2(1.0f));
+  const float2 qp = mul_f2(q, p);
+  const float r0 = -2.0f * ((u0 && q.x < 0.0625f) ? -qp.x : l0), r1 = -2.0f * ((u1 && q.y < 0.0625f) ? -qp.y : l1);
+  float rs0, rs1;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rs0) : "f"(r0));
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rs1) : "f"(r1));
+  const float a0 = r0 * rs0, a1 = r1 * rs1;
+  const float2 th = mul_f2(fma_f2(make_float2((float)x.y, (float)x.w), both2(0x1p-31f), both2(-1.0f)), both2(3.14159265358979323846f));
+  float s, c;
+  __sincosf(th.x, &s, &c);
+  z0 = make_float2(s0 * (-a0 * c), s0 * (-a0 * s));
+  __sincosf(th.y, &s, &c);
+  z1 = make_float2(s1 * (-a1 * c), s1 * (-a1 * s));
 }
 
 // ---------------------------------------------------------------------------

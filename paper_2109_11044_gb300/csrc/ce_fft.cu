@@ -8,9 +8,9 @@
 //           -> T[pair][k1][b];
 //  rows:    P-point FFT along every kept row of T, first m frequencies written
 //           as the Re/Im realizations.
-// For P = 1024 each line is one warp's: 32 points per lane in registers, two
-// in-register 32-point FFTs around a shared-memory transpose.  Other sizes use
-// a shared-memory Stockham radix-4 (final radix-2 stage when log2 P is odd).
+// For P = 1024, 2048 and 4096 each line is 1, 2 or 4 warps': 1024 points per warp, 32
+// per lane in registers, two in-register 32-point FFTs around a shared-memory transpose.
+// Other sizes use a shared-memory Stockham radix-4 (final radix-2 stage when log2 P is odd).
 // Twiddles come from a table computed in FP64 at set-up.
 #include <algorithm>
 
@@ -90,7 +90,7 @@ fft_rowout_kernel(const float2* __restrict__ T, const float2* __restrict__ tw, i
 }
 
 // ---------------------------------------------------------------------------
-// P = 1024: one warp per line, 32 points per lane in registers.  A line x[a]
+// 1024 points in one warp, 32 per lane in registers.  A line x[a]
 // is split as a = t + 32 k (lane t, register k); X[j + 32 l] =
 // sum_t W32^{t l} W1024^{t j} sum_k x[t + 32 k] W32^{k j}: a 32-point FFT in
 // each lane, the twiddles W1024^{t j}, a transpose through shared memory, and
@@ -130,6 +130,8 @@ __host__ __device__ constexpr int brev5(int i) {
 // In-register 32-point forward DFT, natural order in and out (radix-2 DIT).
 // HALF: only the outputs 0..15 are formed (the last stage's differences, which
 // give 16..31, are skipped); v[16..31] are left undefined.
+// A butterfly's sum and difference are one packed instruction each (same roundings as
+// the scalar ones; the passes run out of issue slots before multiply-adders).
 template <bool HALF = false>
 __device__ __forceinline__ void fft32_reg(float2 (&v)[32]) {
 #pragma unroll
@@ -145,8 +147,8 @@ __device__ __forceinline__ void fft32_reg(float2 (&v)[32]) {
       for (int k = 0; k < half; ++k) {
         const float2 a = v[s0 + k];
         const float2 b = mul_w32(v[s0 + k + half], k * (16 / half));
-        v[s0 + k] = make_float2(a.x + b.x, a.y + b.y);
-        if (!(HALF && half == 16)) v[s0 + k + half] = make_float2(a.x - b.x, a.y - b.y);
+        v[s0 + k] = add_f2(a, b);
+        if (!(HALF && half == 16)) v[s0 + k + half] = sub_f2(a, b);
       }
     }
   }
@@ -209,203 +211,159 @@ __device__ __forceinline__ bool warp_bulk_stage(void* dst, const void* src, uint
   return false;
 }
 
-// Column pass with noise, P = 1024.  grid.x = 1024 / 8, grid.y = pairs.
-__global__ void __launch_bounds__(32 * kFastWarps, 3)
-fft1024_colnoise_kernel(const float* __restrict__ sqrt_lam, const float2* __restrict__ tw32, int m,
-                        const __grid_constant__ PhiloxKeys keys, uint32_t pair0, uint32_t event, float2* __restrict__ T,
-                        int* __restrict__ status) {
-  constexpr int P = 1024;
+// Register passes of the ensemble, P = 1024 Q, Q = 1, 2 or 4: Q warps per torus line.  Warp q
+// of a line transforms x_q[t] = x[Q t + q], t < 1024, in registers (the code above); with
+// A_q[j] = W_P^{q j} X_q[j], j < 1024, the line's transform is X[j] = sum_q A_q[j] and, for
+// Q = 4, X[j + 1024] = sum_q (-i)^q A_q[j]: all that the crop keeps, since m <= P / 2.  The
+// A_q pass through the warps' own transpose buffers, whose stride of 1058 keeps the block's
+// reads of neighbouring lines free of bank conflicts, and every warp forms and writes outputs.
+// Bound by instruction issue and the integer and FP32 multipliers in the column pass (88 warp
+// instructions per 32 elements, two thirds of the issue slots used, the multipliers' heavier
+// half 63 % busy) and by the latency of the loads in the row pass.  128 registers a thread
+// (two blocks per SM) keep a batch of twiddles and weights in flight; three blocks of 80 are
+// faster only in the row pass of Q = 1, whose row arrives by bulk copy (50 us against 55, 100 fields).
+// Column / row pass before and now: 32 fields of 2048 x 2048 (P = 4096, before on the
+// shared-memory blocks) 2404 / 1190 us, 1365 / 426; 64 fields of 750 x 750 (P = 2048, before
+// with the even warps forming the outputs) 549 / 179, 467 / 136; 100 fields of 512 x 512
+// (P = 1024, before through a stage with bank conflicts) 211 / 55, 183 / 50.
+constexpr int kLineBuf = 1058;
+
+// v[l] *= W_P^{q (lane + 32 l)}; tw points at the lane's first factor.
+__device__ __forceinline__ void line_twiddle(float2 (&v)[32], const float2* __restrict__ tw, int q) {
+#pragma unroll
+  for (int l = 0; l < 32; ++l) v[l] = cmul(v[l], __ldg(tw + 32 * q * l));
+}
+
+// Column pass with noise.  grid.x = P / (8 / Q), grid.y = pairs.
+template <int Q>
+__global__ void __launch_bounds__(32 * kFastWarps, 2)
+reg_colnoise_kernel(const float* __restrict__ sqrt_lam, const float2* __restrict__ tw, const float2* __restrict__ tw32, int m,
+                    const __grid_constant__ PhiloxKeys keys, uint32_t pair0, uint32_t event, float2* __restrict__ T,
+                    int* __restrict__ status) {
+  constexpr int P = 1024 * Q, L = kFastWarps / Q;
   extern __shared__ __align__(16) float2 smf[];
   __shared__ __align__(8) uint64_t col_bar[kFastWarps];
-  float2* buf = smf + (threadIdx.x >> 5) * (32 * 33);
-  float2* stage = smf;   // [k1][8 columns], reusing the transpose buffers after a barrier
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int b = blockIdx.x * kFastWarps + w;
+  float2* buf = smf + w * kLineBuf;
+  const int b = blockIdx.x * L + w / Q, q = w % Q;
   const int pl = blockIdx.y;
   const uint32_t pair = pair0 + (uint32_t)pl;
-  // the column's 4 KB of weights, staged in the warp's transpose buffer by one bulk copy
-  const float* sl = reinterpret_cast<const float*>(buf);
-  const bool staged = warp_bulk_stage(buf, sqrt_lam + (long long)b * P, P * sizeof(float), &col_bar[w], lane, status);
+  const float* sl = sqrt_lam + (long long)b * P + q;
+  // Q = 1: the column's 4 KB of weights, staged in the warp's transpose buffer by one bulk copy
+  const bool staged = Q > 1 || warp_bulk_stage(buf, sl, P * sizeof(float), &col_bar[w], lane, status);
+  if (Q == 1) sl = reinterpret_cast<const float*>(buf);
   float2 v[32];
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
-    const int a = lane + 32 * k;
-    const uint4 x = philox4x32_10(make_uint4((uint32_t)(a * P + b), pair, 0u, event), keys);
-    const float2 z01 = box_muller(x.x, x.y);
-    const float2 z23 = box_muller(x.z, x.w);
-    const float s0 = staged ? sl[a] : 0.f, s1 = staged ? sl[a + P / 2] : 0.f;
-    v[k] = make_float2(s0 * z01.x, s0 * z01.y);
-    v[k + 16] = make_float2(s1 * z23.x, s1 * z23.y);
+    const int t = lane + 32 * k;   // elements a = Q t + q < P / 2 and a + P / 2 of one counter
+    const uint4 x = philox4x32_10(make_uint4((uint32_t)((Q * t + q) * P + b), pair, 0u, event), keys);
+    const float s0 = staged ? sl[Q * t] : 0.f, s1 = staged ? sl[Q * t + P / 2] : 0.f;
+    box_muller2(x, s0, s1, v[k], v[k + 16]);
   }
   __syncwarp();   // every lane has read its weights before the transpose reuses the buffer
   fft32_reg(v);
-  fft1024_finish<true>(v, buf, tw32, lane);   // outputs kk < m <= 512: l < 16
-  __syncthreads();   // every warp is done with its transpose buffer
+  fft1024_finish<Q == 1>(v, buf, tw32, lane);   // Q = 1: outputs < m <= 512, l < 16
+  const int jm = min(m, 1024);
+  if (Q > 1 && q) line_twiddle(v, tw + q * lane, q);
 #pragma unroll
-  for (int l = 0; l < 16; ++l) {
-    const int kk = lane + 32 * l;
-    if (kk < m) stage[kk * kFastWarps + w] = v[l];
-  }
+  for (int l = 0; l < (Q == 1 ? 16 : 32); ++l)
+    if (lane + 32 * l < jm) buf[lane + 32 * l] = v[l];
   __syncthreads();
-  float2* dst = T + (long long)pl * m * P + blockIdx.x * kFastWarps;
-  for (int e = threadIdx.x; e < m * kFastWarps; e += 32 * kFastWarps) {
-    const int kk = e / kFastWarps, c = e % kFastWarps;
-    dst[(long long)kk * P + c] = stage[e];
+  float2* dst = T + (long long)pl * m * P + blockIdx.x * L;
+#pragma unroll 4
+  for (int e = threadIdx.x; e < jm * L; e += 32 * kFastWarps) {
+    const int j = e / L, c = e % L;
+    const float2* A = smf + c * Q * kLineBuf + j;
+    float2 x = A[0];
+    if (Q == 2) {
+      const float2 o = A[kLineBuf];
+      x = make_float2(x.x + o.x, x.y + o.y);
+    } else if (Q == 4) {
+      const float2 a1 = A[kLineBuf], a2 = A[2 * kLineBuf], a3 = A[3 * kLineBuf];
+      const float2 d = make_float2(x.x - a2.x, x.y - a2.y), f = make_float2(a1.y - a3.y, a3.x - a1.x);   // -i (a1 - a3)
+      x = make_float2((x.x + a2.x) + (a1.x + a3.x), (x.y + a2.y) + (a1.y + a3.y));
+      if (j + 1024 < m) dst[(long long)(j + 1024) * P + c] = make_float2(d.x + f.x, d.y + f.y);
+    }
+    dst[(long long)j * P + c] = x;
   }
 }
 
-// Row pass, P = 1024.  grid.x = ceil(m / 8), grid.y = pairs.  Each warp's row
-// (8 KB) arrives in its transpose buffer by one bulk asynchronous copy, so the
-// load path carries one instruction per row instead of 32 per lane.  The wait
-// is bounded: on expiry the warp sets CE_ERR_TIMEOUT in *status and skips its row.
+// Row pass.  grid.x = ceil(m / (8 / Q)), grid.y = pairs: rows k1 < m of T, the first m
+// frequencies to realizations 2p (real part) and 2p + 1 (imaginary part).  Q = 1: each warp's
+// row (8 KB) arrives in its transpose buffer by one bulk asynchronous copy, so the load path
+// carries one instruction per row instead of 32 per lane; the wait is bounded: on expiry the
+// warp sets CE_ERR_TIMEOUT in *status and skips its row.
 // ACC: add the real parts to realization 2p and subtract the imaginary parts from
 // 2p + 1 (the circulant correction's final conjugation) instead of storing them.
-template <bool ACC = false>
-__global__ void __launch_bounds__(32 * kFastWarps, 3)
-fft1024_rowout_kernel(const float2* __restrict__ T, const float2* __restrict__ tw32, int m, int R_local, int pair_local0,
-                      float* __restrict__ out, int* __restrict__ status) {
-  constexpr int P = 1024;
+template <int Q, bool ACC = false>
+__global__ void __launch_bounds__(32 * kFastWarps, Q > 1 ? 2 : 3)
+reg_rowout_kernel(const float2* __restrict__ T, const float2* __restrict__ tw, const float2* __restrict__ tw32, int m,
+                  int R_local, int pair_local0, float* __restrict__ out, int* __restrict__ status) {
+  constexpr int P = 1024 * Q, L = kFastWarps / Q;
   extern __shared__ __align__(16) float2 smf[];
   __shared__ __align__(8) uint64_t row_bar[kFastWarps];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  float2* buf = smf + w * (32 * 33);
-  const int row = blockIdx.x * kFastWarps + w;
-  if (row >= m) return;
+  float2* buf = smf + w * kLineBuf;
+  const int row = blockIdx.x * L + w / Q, q = w % Q;
   const int pl = blockIdx.y;
-  const float2* src = T + ((long long)pl * m + row) * P;
-  if (!warp_bulk_stage(buf, src, P * sizeof(float2), &row_bar[w], lane, status)) return;
-  float2 v[32];
-#pragma unroll
-  for (int k = 0; k < 32; ++k) v[k] = buf[lane + 32 * k];
-  __syncwarp();   // every lane has its inputs before the transpose reuses the buffer
-  fft32_reg(v);
-  fft1024_finish<true>(v, buf, tw32, lane);   // outputs k2 < m <= 512: l < 16
   const int r_re = 2 * (pair_local0 + pl);
   const bool has_im = r_re + 1 < R_local;
   const long long M = (long long)m * m;
-  float* o_re = out + r_re * M + (long long)row * m;
-#pragma unroll
-  for (int l = 0; l < 16; ++l) {
-    const int k2 = lane + 32 * l;
-    if (k2 < m) {
-      if (ACC) {
-        o_re[k2] += v[l].x;
-        if (has_im) o_re[M + k2] -= v[l].y;
-      } else {
-        o_re[k2] = v[l].x;
-        if (has_im) o_re[M + k2] = v[l].y;
-      }
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------
-// P = 2048: two warps per torus line.  The warp of parity q transforms
-// x_q[t] = x[2t + q], t < 1024, as a 1024-point transform in registers (the
-// code above, with the same 32 x 32 matrix of W1024 twiddles);
-// the line's transform is X[k] = E[k] + W2048^k O[k] for k < 1024, and only the
-// k < m <= 1024 that the crop keeps are formed.  The noise of element a < 1024
-// and a + 1024 comes from one counter (same parity, same warp).
-// ---------------------------------------------------------------------------
-constexpr int kLines2048 = 4;   // torus lines per block of 8 warps
-
-__global__ void __launch_bounds__(256, 2)
-fft2048_colnoise_kernel(const float* __restrict__ sqrt_lam, const float2* __restrict__ tw,
-                        const float2* __restrict__ tw32, int m,
-                        const __grid_constant__ PhiloxKeys keys, uint32_t pair0, uint32_t event, float2* __restrict__ T) {
-  constexpr int P = 2048;
-  extern __shared__ __align__(16) float2 smf[];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  float2* buf = smf + w * (32 * 33);
-  float2* odd = smf + 8 * 32 * 33;   // [line][1024]: W^k O[k]
-  float2* stage = smf;               // [k][line], over the transpose buffers after a barrier
-  const int c = w >> 1, par = w & 1;
-  const int b = blockIdx.x * kLines2048 + c;
-  const int pl = blockIdx.y;
-  const uint32_t pair = pair0 + (uint32_t)pl;
-  const float* sl = sqrt_lam + (long long)b * P;
   float2 v[32];
+  if (Q == 1) {
+    if (row >= m) return;
+    const float2* src = T + ((long long)pl * m + row) * P;
+    if (!warp_bulk_stage(buf, src, P * sizeof(float2), &row_bar[w], lane, status)) return;
 #pragma unroll
-  for (int k = 0; k < 16; ++k) {
-    const int a = 2 * (lane + 32 * k) + par;   // < 1024; a + 1024 is element t + 512
-    const uint4 x = philox4x32_10(make_uint4((uint32_t)(a * P + b), pair, 0u, event), keys);
-    const float2 z01 = box_muller(x.x, x.y);
-    const float2 z23 = box_muller(x.z, x.w);
-    const float s0 = __ldg(sl + a), s1 = __ldg(sl + a + P / 2);
-    v[k] = make_float2(s0 * z01.x, s0 * z01.y);
-    v[k + 16] = make_float2(s1 * z23.x, s1 * z23.y);
+    for (int k = 0; k < 32; ++k) v[k] = buf[lane + 32 * k];
+    __syncwarp();   // every lane has its inputs before the transpose reuses the buffer
+  } else {
+    // rows past the last repeat it (every warp reaches the barrier) and are not written
+    const float2* src = T + ((long long)pl * m + min(row, m - 1)) * P + q;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) v[k] = src[Q * (lane + 32 * k)];
   }
   fft32_reg(v);
-  fft1024_finish(v, buf, tw32, lane);   // lane j holds the transform at j + 32 l in v[l]
-  if (par) {
-#pragma unroll
-    for (int l = 0; l < 32; ++l) {
-      const int k = lane + 32 * l;
-      if (k < m) odd[c * 1024 + k] = cmul(v[l], __ldg(tw + k));
+  fft1024_finish<Q == 1>(v, buf, tw32, lane);
+  auto put = [&](float* o, float2 x) {
+    if (ACC) {
+      o[0] += x.x;
+      if (has_im) o[M] -= x.y;
+    } else {
+      o[0] = x.x;
+      if (has_im) o[M] = x.y;
     }
+  };
+  if (Q == 1) {
+    float* o = out + r_re * M + (long long)row * m;
+#pragma unroll
+    for (int l = 0; l < 16; ++l)
+      if (lane + 32 * l < m) put(o + lane + 32 * l, v[l]);
+    return;
   }
+  const int jm = min(m, 1024);
+  if (q) line_twiddle(v, tw + q * lane, q);
+#pragma unroll
+  for (int l = 0; l < 32; ++l)
+    if (lane + 32 * l < jm) buf[lane + 32 * l] = v[l];
   __syncthreads();
-  if (!par) {
-#pragma unroll
-    for (int l = 0; l < 32; ++l) {
-      const int k = lane + 32 * l;
-      if (k < m) {
-        const float2 o = odd[c * 1024 + k];
-        stage[k * kLines2048 + c] = make_float2(v[l].x + o.x, v[l].y + o.y);
-      }
+  if (row >= m) return;
+  const float2* A0 = smf + (w - q) * kLineBuf;
+  float* o = out + r_re * M + (long long)row * m;
+#pragma unroll 4
+  for (int j = 32 * q + lane; j < jm; j += 32 * Q) {
+    const float2* A = A0 + j;
+    float2 x = A[0];
+    if (Q == 2) {
+      const float2 y = A[kLineBuf];
+      x = make_float2(x.x + y.x, x.y + y.y);
+    } else {
+      const float2 a1 = A[kLineBuf], a2 = A[2 * kLineBuf], a3 = A[3 * kLineBuf];
+      const float2 d = make_float2(x.x - a2.x, x.y - a2.y), f = make_float2(a1.y - a3.y, a3.x - a1.x);   // -i (a1 - a3)
+      x = make_float2((x.x + a2.x) + (a1.x + a3.x), (x.y + a2.y) + (a1.y + a3.y));
+      if (j + 1024 < m) put(o + j + 1024, make_float2(d.x + f.x, d.y + f.y));
     }
-  }
-  __syncthreads();
-  float2* dst = T + (long long)pl * m * P + blockIdx.x * kLines2048;
-  for (int e = threadIdx.x; e < m * kLines2048; e += 256) {
-    const int k = e / kLines2048, cc = e % kLines2048;
-    dst[(long long)k * P + cc] = stage[e];
-  }
-}
-
-// Row pass, P = 2048: rows k1 < m of T, two warps per row; the first m
-// frequencies go to realizations 2p (real part) and 2p + 1 (imaginary part).
-__global__ void __launch_bounds__(256, 2)
-fft2048_rowout_kernel(const float2* __restrict__ T, const float2* __restrict__ tw, const float2* __restrict__ tw32,
-                      int m, int R_local, int pair_local0,
-                      float* __restrict__ out) {
-  constexpr int P = 2048;
-  extern __shared__ __align__(16) float2 smf[];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  float2* buf = smf + w * (32 * 33);
-  float2* odd = smf + 8 * 32 * 33;
-  const int c = w >> 1, par = w & 1;
-  const int row = blockIdx.x * kLines2048 + c;
-  const bool live = row < m;   // every warp reaches the barrier
-  const int pl = blockIdx.y;
-  const float2* src = T + ((long long)pl * m + (live ? row : 0)) * P;
-  float2 v[32];
-#pragma unroll
-  for (int k = 0; k < 32; ++k) v[k] = live ? src[2 * (lane + 32 * k) + par] : make_float2(0.f, 0.f);
-  fft32_reg(v);
-  fft1024_finish(v, buf, tw32, lane);
-  if (par) {
-#pragma unroll
-    for (int l = 0; l < 32; ++l) {
-      const int k = lane + 32 * l;
-      if (k < m) odd[c * 1024 + k] = cmul(v[l], __ldg(tw + k));
-    }
-  }
-  __syncthreads();
-  if (!par && live) {
-    const int r_re = 2 * (pair_local0 + pl);
-    const bool has_im = r_re + 1 < R_local;
-    const long long M = (long long)m * m;
-    float* o_re = out + r_re * M + (long long)row * m;
-#pragma unroll
-    for (int l = 0; l < 32; ++l) {
-      const int k = lane + 32 * l;
-      if (k < m) {
-        const float2 o = odd[c * 1024 + k];
-        o_re[k] = v[l].x + o.x;
-        if (has_im) o_re[M + k] = v[l].y + o.y;
-      }
-    }
+    put(o + j, x);
   }
 }
 
@@ -417,31 +375,17 @@ int launch_ensemble(ce_ctx* ctx, int R, uint64_t seed, uint64_t r_offset, float*
   const uint32_t k0 = (uint32_t)(seed & 0xffffffffu), k1 = (uint32_t)(seed >> 32);
   const uint32_t pair_base = (uint32_t)(r_offset / 2);
   const PhiloxKeys keys = philox_round_keys(k0, k1);
-  if (P == 2048) {
-    // transpose buffers (8 warps) + the odd halves of 4 lines; the output stage reuses the former
-    const size_t shm = sizeof(float2) * ((size_t)8 * 32 * 33 + (size_t)kLines2048 * 1024);
-    CE_CUDA_TRY(cudaFuncSetAttribute(fft2048_colnoise_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-    CE_CUDA_TRY(cudaFuncSetAttribute(fft2048_rowout_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+  if constexpr (P >= 1024 && P <= 4096) {
+    constexpr int Q = P / 1024, L = kFastWarps / Q;
+    const size_t shm = sizeof(float2) * (size_t)kFastWarps * kLineBuf;   // 3 blocks per SM
+    CE_CUDA_TRY(cudaFuncSetAttribute(reg_colnoise_kernel<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+    CE_CUDA_TRY(cudaFuncSetAttribute(reg_rowout_kernel<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
     for (int p0 = 0; p0 < pairs; p0 += chunk) {
       const int np = std::min(chunk, pairs - p0);
-      fft2048_colnoise_kernel<<<dim3(P / kLines2048, np), 256, shm, s>>>(ctx->sqrt_lam_t, ctx->twiddle, ctx->tw32, m, keys,
-                                                                          pair_base + p0, 0u, T);
-      fft2048_rowout_kernel<<<dim3((m + kLines2048 - 1) / kLines2048, np), 256, shm, s>>>(T, ctx->twiddle, ctx->tw32, m,
-                                                                                            R, p0, y);
-      ctx->launches += 2;
-    }
-  } else if (P == 1024) {
-    // m <= P / 2, so the staged columns fit in the transpose buffers; 3 blocks per SM
-    const size_t shm_c = sizeof(float2) * std::max((size_t)kFastWarps * 32 * 33, (size_t)m * kFastWarps);
-    const size_t shm_r = sizeof(float2) * (size_t)kFastWarps * 32 * 33;
-    CE_CUDA_TRY(cudaFuncSetAttribute(fft1024_colnoise_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_c));
-    CE_CUDA_TRY(cudaFuncSetAttribute(fft1024_rowout_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_r));
-    for (int p0 = 0; p0 < pairs; p0 += chunk) {
-      const int np = std::min(chunk, pairs - p0);
-      fft1024_colnoise_kernel<<<dim3(P / kFastWarps, np), 32 * kFastWarps, shm_c, s>>>(ctx->sqrt_lam_t, ctx->tw32, m, keys,
-                                                                                       pair_base + p0, 0u, T, ctx->dev_status);
-      fft1024_rowout_kernel<false><<<dim3((m + kFastWarps - 1) / kFastWarps, np), 32 * kFastWarps, shm_r, s>>>(
-          T, ctx->tw32, m, R, p0, y, ctx->dev_status);
+      reg_colnoise_kernel<Q><<<dim3(P / L, np), 32 * kFastWarps, shm, s>>>(ctx->sqrt_lam_t, ctx->twiddle, ctx->tw32, m, keys,
+                                                                          pair_base + p0, 0u, T, ctx->dev_status);
+      reg_rowout_kernel<Q><<<dim3((m + L - 1) / L, np), 32 * kFastWarps, shm, s>>>(T, ctx->twiddle, ctx->tw32, m, R, p0, y,
+                                                                                  ctx->dev_status);
       ctx->launches += 2;
     }
   } else {
@@ -623,7 +567,7 @@ __global__ void normals_kernel(const uint4* __restrict__ ctr, int count, uint32_
 // forward, times lambda / N, conjugated, and forward again keeping the first m
 // outputs (one kernel, the column stays in registers), rows forward keeping the
 // first m outputs, added to the fields with the final conjugation
-// (fft1024_rowout_kernel<true>).
+// (reg_rowout_kernel<1, true>).
 // ---------------------------------------------------------------------------
 
 // S: pairs x m x m scatter of the weights (pair p: B[2p] + i B[2p+1]); zero first.
@@ -740,7 +684,8 @@ int circulant_correct_1024(ce_ctx* ctx, const float* B, int R, float* y, cudaStr
   const size_t shm = sizeof(float2) * std::max((size_t)kFastWarps * 32 * 33, (size_t)m * (kFastWarps + 1));
   CE_CUDA_TRY(cudaFuncSetAttribute(circ1024_rowfwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
   CE_CUDA_TRY(cudaFuncSetAttribute(circ1024_col_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-  CE_CUDA_TRY(cudaFuncSetAttribute(fft1024_rowout_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+  const size_t shm_r = sizeof(float2) * (size_t)kFastWarps * kLineBuf;
+  CE_CUDA_TRY(cudaFuncSetAttribute(reg_rowout_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_r));
   for (int p0 = 0; p0 < pairs; p0 += chunk) {
     const int np = std::min(chunk, pairs - p0);
     float2* S = ctx->Xc;
@@ -750,8 +695,8 @@ int circulant_correct_1024(ce_ctx* ctx, const float* B, int R, float* y, cudaStr
                                                                               p0, S);
     circ1024_rowfwd_kernel<<<dim3((m + kFastWarps - 1) / kFastWarps, np), 32 * kFastWarps, shm, s>>>(S, m, ctx->tw32, T);
     circ1024_col_kernel<<<dim3(P / kFastWarps, np), 32 * kFastWarps, shm, s>>>(T, m, ctx->sqrt_lam_t, ctx->tw32);
-    fft1024_rowout_kernel<true><<<dim3((m + kFastWarps - 1) / kFastWarps, np), 32 * kFastWarps, shm, s>>>(
-        T, ctx->tw32, m, R, p0, y, ctx->dev_status);
+    reg_rowout_kernel<1, true><<<dim3((m + kFastWarps - 1) / kFastWarps, np), 32 * kFastWarps, shm_r, s>>>(
+        T, ctx->twiddle, ctx->tw32, m, R, p0, y, ctx->dev_status);
     ctx->launches += 4;
   }
   CE_CUDA_TRY(cudaGetLastError());
