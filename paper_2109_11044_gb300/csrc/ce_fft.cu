@@ -132,7 +132,9 @@ __host__ __device__ constexpr int brev5(int i) {
 // give 16..31, are skipped); v[16..31] are left undefined.
 // A butterfly's sum and difference are one packed instruction each (same roundings as
 // the scalar ones; the passes run out of issue slots before multiply-adders).
-template <bool HALF = false>
+// PACKED false: scalar ones (circ1024_col_kernel, whose two transforms around the scaling ran
+// 163 us packed and 116 scalar, 50 fields of 512 x 512).
+template <bool HALF = false, bool PACKED = true>
 __device__ __forceinline__ void fft32_reg(float2 (&v)[32]) {
 #pragma unroll
   for (int i = 0; i < 32; ++i) {
@@ -147,8 +149,8 @@ __device__ __forceinline__ void fft32_reg(float2 (&v)[32]) {
       for (int k = 0; k < half; ++k) {
         const float2 a = v[s0 + k];
         const float2 b = mul_w32(v[s0 + k + half], k * (16 / half));
-        v[s0 + k] = add_f2(a, b);
-        if (!(HALF && half == 16)) v[s0 + k + half] = sub_f2(a, b);
+        v[s0 + k] = PACKED ? add_f2(a, b) : make_float2(a.x + b.x, a.y + b.y);
+        if (!(HALF && half == 16)) v[s0 + k + half] = PACKED ? sub_f2(a, b) : make_float2(a.x - b.x, a.y - b.y);
       }
     }
   }
@@ -159,7 +161,7 @@ __device__ __forceinline__ void fft32_reg(float2 (&v)[32]) {
 // X[j + 32 l] in v[l] (HALF: for l < 16 only).  `tw32` is the 32 x 32 twiddle
 // matrix, tw32[k][t] = W1024^{t k}: each of the 31 loads of a lane reads one row
 // of it contiguously across the warp.
-template <bool HALF = false>
+template <bool HALF = false, bool PACKED = true>
 __device__ __forceinline__ void fft1024_finish(float2 (&v)[32], float2* buf, const float2* __restrict__ tw32, int lane) {
 #pragma unroll
   for (int k = 1; k < 32; ++k) v[k] = cmul(v[k], __ldg(tw32 + k * 32 + lane));
@@ -169,7 +171,7 @@ __device__ __forceinline__ void fft1024_finish(float2 (&v)[32], float2* buf, con
 #pragma unroll
   for (int t = 0; t < 32; ++t) v[t] = buf[lane * 33 + t];
   __syncwarp();
-  fft32_reg<HALF>(v);
+  fft32_reg<HALF, PACKED>(v);
 }
 
 constexpr int kFastWarps = 8;
@@ -294,7 +296,8 @@ reg_colnoise_kernel(const float* __restrict__ sqrt_lam, const float2* __restrict
 // carries one instruction per row instead of 32 per lane; the wait is bounded: on expiry the
 // warp sets CE_ERR_TIMEOUT in *status and skips its row.
 // ACC: add the real parts to realization 2p and subtract the imaginary parts from
-// 2p + 1 (the circulant correction's final conjugation) instead of storing them.
+// 2p + 1 (the circulant correction's final conjugation) instead of storing them; a load per
+// store in turn took 133 us where all loads first take 56 (50 fields of 512 x 512).
 template <int Q, bool ACC = false>
 __global__ void __launch_bounds__(32 * kFastWarps, Q > 1 ? 2 : 3)
 reg_rowout_kernel(const float2* __restrict__ T, const float2* __restrict__ tw, const float2* __restrict__ tw32, int m,
@@ -326,16 +329,22 @@ reg_rowout_kernel(const float2* __restrict__ T, const float2* __restrict__ tw, c
   fft32_reg(v);
   fft1024_finish<Q == 1>(v, buf, tw32, lane);
   auto put = [&](float* o, float2 x) {
-    if (ACC) {
-      o[0] += x.x;
-      if (has_im) o[M] -= x.y;
-    } else {
-      o[0] = x.x;
-      if (has_im) o[M] = x.y;
-    }
+    o[0] = x.x;
+    if (has_im) o[M] = x.y;
   };
   if (Q == 1) {
     float* o = out + r_re * M + (long long)row * m;
+    if (ACC) {   // every load in flight before the first store
+      static_assert(!ACC || Q == 1, "the accumulating form has one warp per row");
+      float2 y[16];
+#pragma unroll
+      for (int l = 0; l < 16; ++l) {
+        const int k = lane + 32 * l;
+        y[l] = make_float2(k < m ? o[k] : 0.f, k < m && has_im ? o[M + k] : 0.f);
+      }
+#pragma unroll
+      for (int l = 0; l < 16; ++l) v[l] = make_float2(y[l].x + v[l].x, y[l].y - v[l].y);
+    }
 #pragma unroll
     for (int l = 0; l < 16; ++l)
       if (lane + 32 * l < m) put(o + lane + 32 * l, v[l]);
@@ -529,14 +538,14 @@ int run_adjoint(ce_ctx* ctx, const float* H, int R, uint64_t seed, uint64_t r_of
   int st = ensure_fft_buffer(ctx, R);
   if (st) return st;
   const int chunk = ensemble_chunk(ctx, R);
+  const uint32_t k0 = (uint32_t)(seed & 0xffffffffu), k1 = (uint32_t)(seed >> 32);
+  const float inv_sigma = (float)(1.0 / ctx->sigma);
   constexpr int CB = FftShape<P>::CB;
   constexpr int ROWS = FftShape<P>::ROWS;
   const size_t shm_c = sizeof(float2) * CB * P;
   const size_t shm_r = sizeof(float2) * ROWS * P;
   CE_CUDA_TRY(cudaFuncSetAttribute(adj_cols_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_c));
   CE_CUDA_TRY(cudaFuncSetAttribute(adj_rows_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_r));
-  const uint32_t k0 = (uint32_t)(seed & 0xffffffffu), k1 = (uint32_t)(seed >> 32);
-  const float inv_sigma = (float)(1.0 / ctx->sigma);
   for (int p0 = 0; p0 < pairs; p0 += chunk) {
     const int np = std::min(chunk, pairs - p0);
     adj_cols_kernel<P><<<dim3((m + CB - 1) / CB, np), FftShape<P>::NT_COLS, shm_c, s>>>(H, m, R, p0, ctx->twiddle, ctx->T);
@@ -630,8 +639,8 @@ circ1024_col_kernel(float2* __restrict__ T, int m, const float* __restrict__ sqr
     v[k] = a < m ? stage[a * LD + w] : make_float2(0.f, 0.f);
   }
   __syncthreads();   // every warp has its column before the transposes reuse the stage
-  fft32_reg(v);
-  fft1024_finish(v, buf, tw32, lane);   // lane j: frequency j + 32 l in v[l]
+  fft32_reg<false, false>(v);
+  fft1024_finish<false, false>(v, buf, tw32, lane);   // lane j: frequency j + 32 l in v[l]
   const float* sl = sqrt_lam_t + (long long)(c0 + w) * P;
   // in groups of eight, each behind a compiler barrier, so that the weights' loads are not
   // all hoisted beside the 64 registers of the line
@@ -646,8 +655,8 @@ circ1024_col_kernel(float2* __restrict__ T, int m, const float* __restrict__ sqr
     }
   }
   asm volatile("" ::: "memory");
-  fft32_reg(v);
-  fft1024_finish<true>(v, buf, tw32, lane);   // outputs j + 32 l < m <= 512: l < 16
+  fft32_reg<false, false>(v);
+  fft1024_finish<true, false>(v, buf, tw32, lane);   // outputs j + 32 l < m <= 512: l < 16
   __syncthreads();   // every warp is done with its transpose buffer
 #pragma unroll
   for (int l = 0; l < 16; ++l) {
