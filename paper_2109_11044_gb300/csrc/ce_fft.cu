@@ -531,6 +531,136 @@ adj_rows_kernel(const float2* __restrict__ T, int m, const float2* __restrict__ 
   }
 }
 
+// The same sums in registers, P = 1024 Q with Q warps per line, rows first.  A field's row is
+// zero past m <= P / 2, so warp r of a line needs no other warp's data: X[Q k + r] is the
+// 1024-point transform of y_r[t] = (x[t] + (-i)^r x[t + 1024]) W_P^{t r} (the second term for
+// Q = 4 only).  Row pass: rows i < m of h to T[pair][i][b], every b.
+template <int Q>
+__device__ __forceinline__ void padded_line_fft(float2 (&v)[32], float2* buf, const float2* __restrict__ tw,
+                                                const float2* __restrict__ tw32, int lane, int r) {
+  if (Q > 1 && r) line_twiddle(v, tw + r * lane, r);
+  fft32_reg(v);
+  fft1024_finish(v, buf, tw32, lane);   // X[Q (lane + 32 l) + r] in v[l]
+}
+template <int Q>
+__device__ __forceinline__ float2 fold_line(float2 x0, float2 x1, int r) {
+  if (Q < 4) return x0;
+  if (r & 1) x1 = make_float2(x1.y, -x1.x);
+  return r & 2 ? sub_f2(x0, x1) : add_f2(x0, x1);
+}
+
+template <int Q>
+__global__ void __launch_bounds__(32 * kFastWarps, 2)
+adj_reg_rows_kernel(const float* __restrict__ H, int m, int R_local, int pair_local0, const float2* __restrict__ tw,
+                    const float2* __restrict__ tw32, float2* __restrict__ T) {
+  constexpr int P = 1024 * Q, L = kFastWarps / Q;
+  extern __shared__ __align__(16) float2 smf[];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, r = w % Q;
+  float2* buf = smf + w * kLineBuf;
+  const int row = blockIdx.x * L + w / Q;
+  const int pl = blockIdx.y;
+  const int r_re = 2 * (pair_local0 + pl);
+  const long long M = (long long)m * m;
+  const bool has_im = r_re + 1 < R_local;
+  // rows past the last repeat it (every warp reaches the barrier) and are not written
+  const float* h = H + r_re * M + (long long)min(row, m - 1) * m;
+  // without a second realization its loads repeat the first's and are dropped: no branch between
+  // the loads, so that all are in flight at once
+  const float* g = has_im ? h + M : h;
+  auto load = [&](int t) {
+    const int i = min(t, m - 1);
+    const float x = __ldg(h + i), y = __ldg(g + i);
+    return make_float2(t < m ? x : 0.f, t < m && has_im ? -y : 0.f);
+  };
+  float2 v[32];
+#pragma unroll
+  for (int k = 0; k < 32; ++k) {
+    const int t = lane + 32 * k;
+    if (Q == 1 && k >= 16) v[k] = make_float2(0.f, 0.f);   // m <= 512
+    else v[k] = fold_line<Q>(load(t), Q == 4 ? load(t + 1024) : make_float2(0.f, 0.f), r);
+  }
+  padded_line_fft<Q>(v, buf, tw, tw32, lane, r);
+#pragma unroll
+  for (int l = 0; l < 32; ++l) buf[lane + 32 * l] = v[l];
+  __syncthreads();
+  if (row >= m) return;
+  const float2* X = smf + (w - r) * kLineBuf;
+  float2* dst = T + ((long long)pl * m + row) * P;
+#pragma unroll 8
+  for (int b = 32 * r + lane; b < P; b += 32 * Q) dst[b] = X[(b % Q) * kLineBuf + b / Q];
+}
+
+// Column pass: columns b of T (m nonzero elements), their transform times the noise, summed.
+// The frequencies a and a + P / 2 of one counter are registers l and l + 16 of one lane.  The
+// weights are read at (b, a) for (a, b): the isotropic embedding (the only one the gradient
+// takes) is symmetric.
+// Bound by instruction issue (noise, two error-free products per element, the transform).
+// Both passes before (shared-memory transforms, columns first, one Philox call per element) and
+// now: 64 fields of 1024 x 1024 (P = 2048) 706 + 1358 us, 204 + 721 (rows with a branch between their loads: 687).
+template <int Q>
+__global__ void __launch_bounds__(32 * kFastWarps, 2)
+adj_reg_cols_kernel(const float2* __restrict__ T, int m, const float2* __restrict__ tw, const float2* __restrict__ tw32,
+                    const float* __restrict__ sqrt_lam, const float* __restrict__ dsdt, float inv_sigma,
+                    const __grid_constant__ PhiloxKeys keys, uint32_t pair0, double* __restrict__ acc) {
+  constexpr int P = 1024 * Q, L = kFastWarps / Q, LD = L + 1;   // LD: an odd stride, no bank conflicts
+  extern __shared__ __align__(16) float2 smf[];
+  __shared__ double red[2][kFastWarps];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, r = w % Q, c = w / Q;
+  float2* buf = smf + w * kLineBuf;
+  const int b = blockIdx.x * L + c;
+  const int pl = blockIdx.y;
+  const float2* src = T + (long long)pl * m * P + blockIdx.x * L;
+#pragma unroll 8
+  for (int e = threadIdx.x; e < m * L; e += 32 * kFastWarps)
+    smf[(e / L) * LD + e % L] = src[(long long)(e / L) * P + e % L];
+  __syncthreads();
+  auto load = [&](int t) { return t < m ? smf[t * LD + c] : make_float2(0.f, 0.f); };
+  float2 v[32];
+#pragma unroll
+  for (int k = 0; k < 32; ++k) {
+    const int t = lane + 32 * k;
+    if (Q == 1 && k >= 16) v[k] = make_float2(0.f, 0.f);
+    else v[k] = fold_line<Q>(load(t), Q == 4 ? load(t + 1024) : make_float2(0.f, 0.f), r);
+  }
+  __syncthreads();   // every warp has its column before the transposes reuse the buffers
+  padded_line_fft<Q>(v, buf, tw, tw32, lane, r);
+  // sums as FP32 pairs with error-free transformations
+  float2 pt = make_float2(0.f, 0.f), ps = make_float2(0.f, 0.f);
+  auto add_product = [](float2& a, float x, float y) {
+    const float p = __fmul_rn(x, y), pe = fmaf(x, y, -p);
+    const float t = __fadd_rn(a.x, p), z = __fsub_rn(t, a.x);
+    a.y += __fadd_rn(__fsub_rn(a.x, __fsub_rn(t, z)), __fsub_rn(p, z)) + pe;
+    a.x = t;
+  };
+  const float* sl = sqrt_lam + (long long)b * P + r;
+  const float* dl = dsdt + (long long)b * P + r;
+#pragma unroll
+  for (int l = 0; l < 16; ++l) {
+    const int k = Q * (lane + 32 * l);   // frequency a = k + r < P / 2
+    const uint4 x = philox4x32_10(make_uint4((uint32_t)((k + r) * P + b), pair0 + (uint32_t)pl, 0u, 0u), keys);
+    float2 z0, z1;
+    box_muller2(x, 1.f, 1.f, z0, z1);
+    const float re0 = z0.x * v[l].x - z0.y * v[l].y, re1 = z1.x * v[l + 16].x - z1.y * v[l + 16].y;
+    add_product(pt, __ldg(dl + k), re0);
+    add_product(pt, __ldg(dl + k + P / 2), re1);
+    add_product(ps, __ldg(sl + k) * inv_sigma, re0);
+    add_product(ps, __ldg(sl + k + P / 2) * inv_sigma, re1);
+  }
+  double st = (double)pt.x + (double)pt.y, ss = (double)ps.x + (double)ps.y;
+  for (int o = 16; o; o >>= 1) {
+    st += __shfl_xor_sync(0xffffffffu, st, o);
+    ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  }
+  if (lane == 0) { red[0][w] = st; red[1][w] = ss; }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t0 = 0.0, t1 = 0.0;
+    for (int i = 0; i < kFastWarps; ++i) { t0 += red[0][i]; t1 += red[1][i]; }
+    atomicAdd(acc + 0, t0);
+    atomicAdd(acc + 1, t1);
+  }
+}
+
 template <int P>
 int run_adjoint(ce_ctx* ctx, const float* H, int R, uint64_t seed, uint64_t r_offset, double* acc, cudaStream_t s) {
   const int m = ctx->m;
@@ -540,17 +670,31 @@ int run_adjoint(ce_ctx* ctx, const float* H, int R, uint64_t seed, uint64_t r_of
   const int chunk = ensemble_chunk(ctx, R);
   const uint32_t k0 = (uint32_t)(seed & 0xffffffffu), k1 = (uint32_t)(seed >> 32);
   const float inv_sigma = (float)(1.0 / ctx->sigma);
-  constexpr int CB = FftShape<P>::CB;
-  constexpr int ROWS = FftShape<P>::ROWS;
-  const size_t shm_c = sizeof(float2) * CB * P;
-  const size_t shm_r = sizeof(float2) * ROWS * P;
-  CE_CUDA_TRY(cudaFuncSetAttribute(adj_cols_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_c));
-  CE_CUDA_TRY(cudaFuncSetAttribute(adj_rows_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_r));
-  for (int p0 = 0; p0 < pairs; p0 += chunk) {
-    const int np = std::min(chunk, pairs - p0);
-    adj_cols_kernel<P><<<dim3((m + CB - 1) / CB, np), FftShape<P>::NT_COLS, shm_c, s>>>(H, m, R, p0, ctx->twiddle, ctx->T);
-    adj_rows_kernel<P><<<dim3(P / ROWS, np), FftShape<P>::NT_ROWS, shm_r, s>>>(
-        ctx->T, m, ctx->twiddle, ctx->sqrt_lam, ctx->ds_theta, inv_sigma, k0, k1, (uint32_t)(r_offset / 2) + p0, acc);
+  if constexpr (P >= 1024 && P <= 4096) {
+    constexpr int Q = P / 1024, L = kFastWarps / Q;
+    const size_t shm = sizeof(float2) * (size_t)kFastWarps * kLineBuf;   // holds m x (L + 1) staged elements too
+    const PhiloxKeys keys = philox_round_keys(k0, k1);
+    CE_CUDA_TRY(cudaFuncSetAttribute(adj_reg_rows_kernel<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+    CE_CUDA_TRY(cudaFuncSetAttribute(adj_reg_cols_kernel<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+    for (int p0 = 0; p0 < pairs; p0 += chunk) {
+      const int np = std::min(chunk, pairs - p0);
+      adj_reg_rows_kernel<Q><<<dim3((m + L - 1) / L, np), 32 * kFastWarps, shm, s>>>(H, m, R, p0, ctx->twiddle, ctx->tw32, ctx->T);
+      adj_reg_cols_kernel<Q><<<dim3(P / L, np), 32 * kFastWarps, shm, s>>>(
+          ctx->T, m, ctx->twiddle, ctx->tw32, ctx->sqrt_lam, ctx->ds_theta, inv_sigma, keys, (uint32_t)(r_offset / 2) + p0, acc);
+    }
+  } else {
+    constexpr int CB = FftShape<P>::CB;
+    constexpr int ROWS = FftShape<P>::ROWS;
+    const size_t shm_c = sizeof(float2) * CB * P;
+    const size_t shm_r = sizeof(float2) * ROWS * P;
+    CE_CUDA_TRY(cudaFuncSetAttribute(adj_cols_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_c));
+    CE_CUDA_TRY(cudaFuncSetAttribute(adj_rows_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_r));
+    for (int p0 = 0; p0 < pairs; p0 += chunk) {
+      const int np = std::min(chunk, pairs - p0);
+      adj_cols_kernel<P><<<dim3((m + CB - 1) / CB, np), FftShape<P>::NT_COLS, shm_c, s>>>(H, m, R, p0, ctx->twiddle, ctx->T);
+      adj_rows_kernel<P><<<dim3(P / ROWS, np), FftShape<P>::NT_ROWS, shm_r, s>>>(
+          ctx->T, m, ctx->twiddle, ctx->sqrt_lam, ctx->ds_theta, inv_sigma, k0, k1, (uint32_t)(r_offset / 2) + p0, acc);
+    }
   }
   CE_CUDA_TRY(cudaGetLastError());
   return CE_OK;
