@@ -33,43 +33,74 @@ __global__ void embed_kernel(double2* __restrict__ buf, int P, double h, double 
   buf[e] = make_double2(0.5 * (c1 + c2), 0.0);
 }
 
-// One radix-2 Stockham FFT (forward, unnormalised) of length P per block, in
+// tw[k] = e^{-2 pi i k / P}, k < P / 2.
+__global__ void twiddle64_kernel(double2* __restrict__ tw, int half) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= half) return;
+  double s, c;
+  sincospi(-(double)k / (double)half, &s, &c);
+  tw[k] = make_double2(c, s);
+}
+
+// One radix-2 Stockham FFT (forward, unnormalised) of length P = 2^logP per block, in
 // shared memory.  Line `blockIdx.x` starts at buf + blockIdx.x * line_stride and
 // its elements are elem_stride apart.  Each stage reads all of a thread's
 // butterfly inputs into registers before any thread overwrites the line.
+// Bound by FP64 arithmetic (two multiply-adds per SM and clock): a butterfly is 8 operations, so
+// its factor comes from a table (the same bits as an evaluation in place, k / Ns and
+// k (P / 2 Ns) / (P / 2) being the same number), not from a sine and cosine of its own, which
+// cost several times that: six passes over 512 x 512 took 849 us, now 148.
 constexpr int kFft64Threads = 1024;
 constexpr int kFft64MaxB = 4;   // P <= 8192
 
 __global__ void __launch_bounds__(kFft64Threads)
-fft64_lines(double2* __restrict__ buf, int P, long long line_stride, long long elem_stride) {
+fft64_lines(double2* __restrict__ buf, int logP, long long line_stride, long long elem_stride, const double2* __restrict__ tw) {
   extern __shared__ double2 sm64[];
+  const int P = 1 << logP, half = P / 2;
   double2* line = buf + (long long)blockIdx.x * line_stride;
   for (int e = threadIdx.x; e < P; e += blockDim.x) sm64[e] = line[(long long)e * elem_stride];
   __syncthreads();
-  const int half = P / 2;
-  for (int Ns = 1; Ns < P; Ns *= 2) {
+  for (int l = 0; l < logP; ++l) {
+    const int Ns = 1 << l;
     double2 v0[kFft64MaxB], v1[kFft64MaxB];
-    int nb = 0;
-    for (int j = threadIdx.x; j < half; j += blockDim.x, ++nb) {
-      const int k = j % Ns;
+#pragma unroll
+    for (int t = 0; t < kFft64MaxB; ++t) {
+      const int j = threadIdx.x + t * blockDim.x;
+      if (j >= half) break;
+      const int k = j & (Ns - 1);
       const double2 a = sm64[j], b = sm64[j + half];
-      double s, c;
-      sincospi(-(double)k / (double)Ns, &s, &c);   // e^{-2 pi i k / (2 Ns)}
-      const double2 bw = make_double2(b.x * c - b.y * s, b.x * s + b.y * c);
-      v0[nb] = make_double2(a.x + bw.x, a.y + bw.y);
-      v1[nb] = make_double2(a.x - bw.x, a.y - bw.y);
+      const double2 w = __ldg(tw + ((long long)k << (logP - 1 - l)));   // e^{-2 pi i k / (2 Ns)}
+      const double2 bw = make_double2(b.x * w.x - b.y * w.y, b.x * w.y + b.y * w.x);
+      v0[t] = make_double2(a.x + bw.x, a.y + bw.y);
+      v1[t] = make_double2(a.x - bw.x, a.y - bw.y);
     }
     __syncthreads();
-    nb = 0;
-    for (int j = threadIdx.x; j < half; j += blockDim.x, ++nb) {
-      const int k = j % Ns;
-      const int base = (j / Ns) * 2 * Ns + k;
-      sm64[base] = v0[nb];
-      sm64[base + Ns] = v1[nb];
+#pragma unroll
+    for (int t = 0; t < kFft64MaxB; ++t) {
+      const int j = threadIdx.x + t * blockDim.x;
+      if (j >= half) break;
+      const int k = j & (Ns - 1);
+      const int base = ((j >> l) << (l + 1)) + k;
+      sm64[base] = v0[t];
+      sm64[base + Ns] = v1[t];
     }
     __syncthreads();
   }
   for (int e = threadIdx.x; e < P; e += blockDim.x) line[(long long)e * elem_stride] = sm64[e];
+}
+
+// The two-dimensional transform of the P x P array buf, rows then columns; tw (P / 2 elements)
+// is filled here.
+int fft64_square(double2* buf, int P, double2* tw, bool fill, cudaStream_t s) {
+  const size_t shm = sizeof(double2) * P;
+  CE_CUDA_TRY(cudaFuncSetAttribute(fft64_lines, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+  const int thr = P / 2 < kFft64Threads ? P / 2 : kFft64Threads;
+  int logP = 0;
+  while ((1 << logP) < P) ++logP;
+  if (fill) twiddle64_kernel<<<(P / 2 + 255) / 256, 256, 0, s>>>(tw, P / 2);
+  fft64_lines<<<P, thr, shm, s>>>(buf, logP, P, 1, tw);
+  fft64_lines<<<P, thr, shm, s>>>(buf, logP, 1, P, tw);
+  return CE_OK;
 }
 
 // Per-block min and max of the real parts.
@@ -170,18 +201,15 @@ __global__ void twiddle32_kernel(float2* __restrict__ tw32) {
 int eigs_dsqrt_dtheta(ce_ctx* ctx, float* ds, cudaStream_t s) {
   const int P = ctx->P;
   const long long N = (long long)P * P;
-  double2* lam = (double2*)dalloc(ctx, sizeof(double2) * N);
+  double2* lam = (double2*)dalloc(ctx, sizeof(double2) * (N + P / 2));   // and the transform's factors
   double2* dlam = (double2*)dalloc(ctx, sizeof(double2) * N);
   if (!lam || !dlam) { dfree(ctx, lam); dfree(ctx, dlam); return fail(ctx, CE_ERR_OOM, "embedding derivative"); }
   embed_pair_kernel<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(lam, dlam, P, ctx->h, ctx->sigma * ctx->sigma, ctx->range,
                                                                ctx->nu == 1.5 ? 1 : 0);
-  const size_t shm = sizeof(double2) * P;
-  CE_CUDA_TRY(cudaFuncSetAttribute(fft64_lines, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-  const int thr = P / 2 < kFft64Threads ? P / 2 : kFft64Threads;
-  for (double2* buf : {lam, dlam}) {
-    fft64_lines<<<P, thr, shm, s>>>(buf, P, P, 1);
-    fft64_lines<<<P, thr, shm, s>>>(buf, P, 1, P);
-  }
+  double2* tw = lam + N;
+  int st = fft64_square(lam, P, tw, true, s);
+  if (st == CE_OK) st = fft64_square(dlam, P, tw, false, s);
+  if (st) { dfree(ctx, lam); dfree(ctx, dlam); return st; }
   dsqrt_kernel<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(lam, dlam, N, ds);
   CE_CUDA_TRY(cudaGetLastError());
   CE_CUDA_TRY(cudaStreamSynchronize(s));
@@ -198,16 +226,12 @@ int eigs_setup(ce_ctx* ctx, int max_growth, cudaStream_t s) {
   for (int g = 0; g <= max_growth; ++g, P *= 2) {
     if (P > 8192) return fail(ctx, CE_ERR_EMBED, "embedding would exceed 8192 x 8192");
     const long long N = (long long)P * P;
-    double2* buf = (double2*)dalloc(ctx, sizeof(double2) * N);
+    double2* buf = (double2*)dalloc(ctx, sizeof(double2) * (N + P / 2));   // and the transform's factors
     double* mm = (double*)dalloc(ctx, sizeof(double) * 2 * 1024);
     if (!buf || !mm) { dfree(ctx, buf); dfree(ctx, mm); return fail(ctx, CE_ERR_OOM, "embedding buffer"); }
     embed_kernel<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(buf, P, ctx->h, sigma2, ctx->range, nu3,
                                                               make_aniso(ctx->aniso_ratio, ctx->aniso_angle));
-    const size_t shm = sizeof(double2) * P;
-    CE_CUDA_TRY(cudaFuncSetAttribute(fft64_lines, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-    const int thr = P / 2 < kFft64Threads ? P / 2 : kFft64Threads;
-    fft64_lines<<<P, thr, shm, s>>>(buf, P, P, 1);   // rows
-    fft64_lines<<<P, thr, shm, s>>>(buf, P, 1, P);   // columns
+    if (const int st = fft64_square(buf, P, buf + N, true, s)) { dfree(ctx, buf); dfree(ctx, mm); return st; }
     minmax_kernel<<<1024, 256, 0, s>>>(buf, N, mm);
     CE_CUDA_TRY(cudaGetLastError());
     std::vector<double> h_mm(2 * 1024);
