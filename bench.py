@@ -42,13 +42,13 @@ METRIC = "conditional realizations/s at 512^2 grid, n=2000 obs, R=100"
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch of the f16x3 tensor-core
 # correction on the 512^2 x 2000-site x R=100 workload (profiles/correct_tc_shakemap512.md);
 # None while the kernel has changed since the last capture
-CORRECT_TC_DRAM_BYTES = None   # last capture (150.6 MB) predates the double-buffered cross accumulator
+CORRECT_TC_DRAM_BYTES = None   # last capture (150.6 MB) predates the packed producers
 FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0}
 # Warp instructions of the two P = 1024 ensemble passes per realization pair
 # (smsp__inst_executed.sum of one launch of each pass over its pairs;
 # profiles/fft1024_colnoise_shakemap512.md, fft1024_rowout_shakemap512.md): column
 # pass with the noise, row pass
-FFT1024_WARP_INSTR_PER_PAIR = (44.190568e6 / 13, 9.220123e6 / 13)
+FFT1024_WARP_INSTR_PER_PAIR = (37.074215e6 / 13, 7.077946e6 / 13)
 
 
 def peaks():
@@ -937,7 +937,7 @@ def main():
               "useful_tflops": se_flops / (se_ms / 1e3) / 1e12, "peak_fp32_tflops": fp32_peak,
               "peak_source": "measured FP32 FMA rate (ce_unit_rates)",
               "frac": se_flops / (se_ms / 1e3) / 1e12 / fp32_peak,
-              "note": "FP32 CUDA-core products with the hi/lo pair issue 2x the useful flops; "
+              "note": "one of the two products in FP32 with the hi/lo pair (2x the useful flops), one from exact digits; "
                       "includes the per-call work-buffer allocation"}
 
     # the other workloads: the precision forms at 2048^2, the 64-event batch, the gradient at 1024^2

@@ -127,9 +127,10 @@ int ce_setup(ce_ctx** out, const ce_grid* grid, const ce_cov* cov, int max_growt
  * CE_NN (Section 2.2, Section 3.2): the union J_N of each site's k nearest grid
  * nodes, the surrogate-data map K_No A^-1, the surrogate variances sigma_N^2 and
  * the prediction matrix K_NN + tau^2 I + diag(sigma_N^2).
- * The prediction matrix is factored by an FP64 Cholesky on the device
- * (CE_ERR_NOT_SPD if that fails) and inverted in FP64; the inverse is kept as
- * an FP32 pair (hi + lo).  Synchronises the stream.  May be called again to
+ * The prediction matrix is inverted in FP64 on the device by symmetric block
+ * sweeps (CE_ERR_NOT_SPD if a pivot, those of its Cholesky factor, is not
+ * positive); the inverse is kept as an FP32 pair (hi + lo), from 1800 rows on
+ * also as 8-bit digits.  Synchronises the stream.  May be called again to
  * replace the sites.
  * ------------------------------------------------------------------------- */
 int ce_krige_weights(ce_ctx* ctx, const double* obs_xy, int n, const ce_nbhd* nb);
@@ -240,12 +241,12 @@ int ce_set_box_joint(ce_ctx* ctx, int on, int* n_boxes);
  * diagonal of (I - W_2 S) K_gg (I - W_2 S)^T + W_2 D W_2^T (Section 3.1) with
  * S = W_1 and D the synthetic-noise covariance (diag phi^2, or the grid-box
  * blocks of ce_set_box_joint) in local mode, and the surrogate model's
- * sigma^2 - k_g^T A_N^-1 k_g (Section 3.2) in NN mode.  FP64 covariance
- * evaluation, FP32 products with the stored inverse pair, FP64 sums per node.
- * CE_ERR_STATE while a trend is set.  Cost in local mode: two FP32 products of
- * M x n by n x n, plus n^2 K^2 / 2 FP64 multiply-adds to form Q (K = (2 np)^2
- * window nodes; about 4 ms at n = 2000, K = 36, but minutes at n = 10000,
- * K = 64).  Allocates its work buffers (about 300 MB
+ * sigma^2 - k_g^T A_N^-1 k_g (Section 3.2) in NN mode.  Covariances as FP32
+ * pairs, FP32 products with the stored inverse pair, Q by integer window sums and
+ * its product from exact digits, FP64 sums per node.
+ * CE_ERR_STATE while a trend is set.  Cost in local mode: two products of
+ * M x n by n x n (M grid nodes; 177 ms in all at 512 x 512, n = 2000, 36 window
+ * nodes).  Allocates its work buffers (about 300 MB
  * at most, plus n x n pairs and an m x (2m - 1) table) and synchronises `stream`. */
 int ce_se_map(ce_ctx* ctx, float* se_exact_dev, float* se_approx_dev, void* stream);
 
@@ -415,7 +416,7 @@ int ce_condsim_grad(ce_ctx* ctx, const float* z_dev, int R, uint64_t seed, uint6
  * Eq. (condmvn) (z ~ N(0, A), A = K_oo + tau^2 I):
  *   *out = -z^T A^-1 z / 2 - log det A / 2 - (n/2) log(2 pi).
  * z_dev: device float32, n values in the caller's site order.  Uses the FP64
- * log-determinant of the set-up's Cholesky factor and the stored inverse pair
+ * log-determinant from the set-up's pivots and the stored inverse pair
  * (hi + lo), with the quadratic form summed in FP64 on the device.  Local
  * Kriging set-up only and no trend (CE_ERR_STATE otherwise: the NN context
  * factors its surrogate matrix instead of A).  Allocates a buffer of n floats

@@ -2,7 +2,7 @@
 // z ~ N(0, A) with A = K_oo + tau^2 I, so
 //   l = -z^T A^-1 z / 2 - log det A / 2 - (n / 2) log(2 pi).
 // The context holds A^-1 as an FP32 pair (hi + lo, internal site order) and
-// log det A from the FP64 Cholesky factor of its set-up; the quadratic form is
+// log det A from the FP64 pivots of its set-up; the quadratic form is
 // summed here in FP64, one warp per row of A^-1.
 #include <cmath>
 
