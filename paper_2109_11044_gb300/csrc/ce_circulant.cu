@@ -148,10 +148,10 @@ int run_circulant(ce_ctx* ctx, const float* B, int R, float* y, cudaStream_t s) 
   const int pairs = (R + 1) / 2;
   const int chunk = ctx->circ_pairs;
   const size_t shm_c = sizeof(float2) * CB * P, shm_r = sizeof(float2) * ROWS * P;
-  CE_CUDA_TRY(cudaFuncSetAttribute(circ_colfwd_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_c));
-  CE_CUDA_TRY(cudaFuncSetAttribute(circ_colinv_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_c));
-  CE_CUDA_TRY(cudaFuncSetAttribute(circ_rowfwd_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_r));
-  CE_CUDA_TRY(cudaFuncSetAttribute(circ_rowinv_add_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_r));
+  CE_CUDA_TRY(set_max_smem(circ_colfwd_kernel<P>, shm_c));
+  CE_CUDA_TRY(set_max_smem(circ_colinv_kernel<P>, shm_c));
+  CE_CUDA_TRY(set_max_smem(circ_rowfwd_kernel<P>, shm_r));
+  CE_CUDA_TRY(set_max_smem(circ_rowinv_add_kernel<P>, shm_r));
   for (int p0 = 0; p0 < pairs; p0 += chunk) {
     const int np = std::min(chunk, pairs - p0);
     CE_CUDA_TRY(cudaMemsetAsync(ctx->Xc, 0, sizeof(float2) * (size_t)np * P * P, s));

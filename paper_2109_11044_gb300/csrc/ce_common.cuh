@@ -17,6 +17,14 @@ namespace ce {
 
 int cuda_fail(cudaError_t e, const char* what, const char* file, int line);
 
+// Allow a kernel up to `bytes` of dynamic shared memory.  The limit belongs to the process and
+// a launch above it fails, so `bytes` is a constant of the kernel (the most that any call of it
+// asks for), never a call's own size: another thread's call may come between this and the launch.
+template <typename Kernel>
+inline cudaError_t set_max_smem(Kernel kernel, size_t bytes) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 // ---------------------------------------------------------------------------
 // Philox4x32-10 (Salmon, Moraes, Dror & Shaw, SC'11): ten rounds of two 32x32
 // multiplications with the key advanced by the Weyl constants between rounds.

@@ -444,7 +444,7 @@ int launch_correct(ce_ctx* ctx, const float* B, int R, float* y, cudaStream_t s)
     const int tn = fills(tn0) ? tn0 : (fills(tn1) ? tn1 : tn2);
     auto kernel = tn == tn0 ? k0 : (tn == tn1 ? k1 : k2);
     const size_t smem = sizeof(float) * 2 * KC * (size_t)(tn + rtile);
-    CE_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CE_CUDA_TRY(set_max_smem(kernel, smem));
     kernel<<<dim3((unsigned)((M + tn - 1) / tn), (unsigned)rb), nthreads, smem, s>>>(y, ctx->m, ctx->obs, ctx->nobs, Bk, ldr, ldk, R,
                                                                                   mf, an, a22);
     return CE_OK;

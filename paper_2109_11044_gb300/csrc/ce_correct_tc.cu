@@ -51,6 +51,7 @@ MaternF matern_grid_units(const ce_ctx* ctx);
 namespace {
 
 constexpr int TM = 128;            // nodes per tile (MMA M)
+constexpr uint32_t kTcSmem = 224 * 1024;   // most dynamic shared memory of a block
 // A row of a chunk is 128 bytes of operands, so a chunk holds 64 sites of a 16-bit kind
 // or 32 of tf32, and each MMA takes 32 bytes of K (16 or 8 sites).
 template <int KIND> struct Op {
@@ -787,8 +788,7 @@ __global__ void absmax_kernel(const float* __restrict__ B, int ldb, int R, int n
 
 template <int NPW, int KIND, bool NU3, bool ANISO = false, bool MULTI = false, bool AMEM = false>
 int launch_tc(const TcArgs& a, size_t smem, cudaStream_t s) {
-  CE_CUDA_TRY(cudaFuncSetAttribute(correct_tc_kernel<NPW, KIND, NU3, ANISO, MULTI, AMEM>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  CE_CUDA_TRY(set_max_smem(correct_tc_kernel<NPW, KIND, NU3, ANISO, MULTI, AMEM>, kTcSmem));
   int nsm = 0, dev = 0;
   CE_CUDA_TRY(cudaGetDevice(&dev));
   CE_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -958,7 +958,7 @@ int tc_launch(ce_ctx* owner, TcEvent* ev, int nev, int kind, int Npad, bool nu3,
   a.stage_bytes = 32768u + a.bblock;
   // the epilogue's running sums (128 rows x Npad FP32) after the stages
   const uint32_t run_bytes = 128u * 4u * (uint32_t)Npad;
-  const uint32_t budget = 224u * 1024u - 1024u - run_bytes;
+  const uint32_t budget = kTcSmem - 1024u - run_bytes;
   a.stages = (int)(budget / a.stage_bytes);
   if (a.stages > 4) a.stages = 4;
   if (a.stages < 2) return fail(owner, CE_ERR_ARG, "tensor-core stage does not fit in shared memory");

@@ -51,7 +51,8 @@ __global__ void twiddle64_kernel(double2* __restrict__ tw, int half) {
 // k (P / 2 Ns) / (P / 2) being the same number), not from a sine and cosine of its own, which
 // cost several times that: six passes over 512 x 512 took 849 us, now 148.
 constexpr int kFft64Threads = 1024;
-constexpr int kFft64MaxB = 4;   // P <= 8192
+constexpr int kFft64MaxB = 4;
+constexpr int kFft64MaxP = 2 * kFft64MaxB * kFft64Threads;   // 8192
 
 __global__ void __launch_bounds__(kFft64Threads)
 fft64_lines(double2* __restrict__ buf, int logP, long long line_stride, long long elem_stride, const double2* __restrict__ tw) {
@@ -93,7 +94,7 @@ fft64_lines(double2* __restrict__ buf, int logP, long long line_stride, long lon
 // is filled here.
 int fft64_square(double2* buf, int P, double2* tw, bool fill, cudaStream_t s) {
   const size_t shm = sizeof(double2) * P;
-  CE_CUDA_TRY(cudaFuncSetAttribute(fft64_lines, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+  CE_CUDA_TRY(set_max_smem(fft64_lines, sizeof(double2) * kFft64MaxP));
   const int thr = P / 2 < kFft64Threads ? P / 2 : kFft64Threads;
   int logP = 0;
   while ((1 << logP) < P) ++logP;

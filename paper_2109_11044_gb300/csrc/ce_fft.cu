@@ -387,8 +387,8 @@ int launch_ensemble(ce_ctx* ctx, int R, uint64_t seed, uint64_t r_offset, float*
   if constexpr (P >= 1024 && P <= 4096) {
     constexpr int Q = P / 1024, L = kFastWarps / Q;
     const size_t shm = sizeof(float2) * (size_t)kFastWarps * kLineBuf;   // 3 blocks per SM
-    CE_CUDA_TRY(cudaFuncSetAttribute(reg_colnoise_kernel<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-    CE_CUDA_TRY(cudaFuncSetAttribute(reg_rowout_kernel<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+    CE_CUDA_TRY(set_max_smem(reg_colnoise_kernel<Q>, shm));
+    CE_CUDA_TRY(set_max_smem(reg_rowout_kernel<Q>, shm));
     for (int p0 = 0; p0 < pairs; p0 += chunk) {
       const int np = std::min(chunk, pairs - p0);
       reg_colnoise_kernel<Q><<<dim3(P / L, np), 32 * kFastWarps, shm, s>>>(ctx->sqrt_lam_t, ctx->twiddle, ctx->tw32, m, keys,
@@ -402,8 +402,8 @@ int launch_ensemble(ce_ctx* ctx, int R, uint64_t seed, uint64_t r_offset, float*
     constexpr int ROWS = FftShape<P>::ROWS;
     const size_t shm_c = sizeof(float2) * CB * P;
     const size_t shm_r = sizeof(float2) * ROWS * P;
-    CE_CUDA_TRY(cudaFuncSetAttribute(fft_colnoise_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_c));
-    CE_CUDA_TRY(cudaFuncSetAttribute(fft_rowout_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_r));
+    CE_CUDA_TRY(set_max_smem(fft_colnoise_kernel<P>, shm_c));
+    CE_CUDA_TRY(set_max_smem(fft_rowout_kernel<P>, shm_r));
     for (int p0 = 0; p0 < pairs; p0 += chunk) {
       const int np = std::min(chunk, pairs - p0);
       fft_colnoise_kernel<P><<<dim3(P / CB, np), FftShape<P>::NT_COLS, shm_c, s>>>(ctx->sqrt_lam_t, ctx->twiddle, m, keys,
@@ -674,8 +674,8 @@ int run_adjoint(ce_ctx* ctx, const float* H, int R, uint64_t seed, uint64_t r_of
     constexpr int Q = P / 1024, L = kFastWarps / Q;
     const size_t shm = sizeof(float2) * (size_t)kFastWarps * kLineBuf;   // holds m x (L + 1) staged elements too
     const PhiloxKeys keys = philox_round_keys(k0, k1);
-    CE_CUDA_TRY(cudaFuncSetAttribute(adj_reg_rows_kernel<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-    CE_CUDA_TRY(cudaFuncSetAttribute(adj_reg_cols_kernel<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+    CE_CUDA_TRY(set_max_smem(adj_reg_rows_kernel<Q>, shm));
+    CE_CUDA_TRY(set_max_smem(adj_reg_cols_kernel<Q>, shm));
     for (int p0 = 0; p0 < pairs; p0 += chunk) {
       const int np = std::min(chunk, pairs - p0);
       adj_reg_rows_kernel<Q><<<dim3((m + L - 1) / L, np), 32 * kFastWarps, shm, s>>>(H, m, R, p0, ctx->twiddle, ctx->tw32, ctx->T);
@@ -687,8 +687,8 @@ int run_adjoint(ce_ctx* ctx, const float* H, int R, uint64_t seed, uint64_t r_of
     constexpr int ROWS = FftShape<P>::ROWS;
     const size_t shm_c = sizeof(float2) * CB * P;
     const size_t shm_r = sizeof(float2) * ROWS * P;
-    CE_CUDA_TRY(cudaFuncSetAttribute(adj_cols_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_c));
-    CE_CUDA_TRY(cudaFuncSetAttribute(adj_rows_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_r));
+    CE_CUDA_TRY(set_max_smem(adj_cols_kernel<P>, shm_c));
+    CE_CUDA_TRY(set_max_smem(adj_rows_kernel<P>, shm_r));
     for (int p0 = 0; p0 < pairs; p0 += chunk) {
       const int np = std::min(chunk, pairs - p0);
       adj_cols_kernel<P><<<dim3((m + CB - 1) / CB, np), FftShape<P>::NT_COLS, shm_c, s>>>(H, m, R, p0, ctx->twiddle, ctx->T);
@@ -834,11 +834,12 @@ int circulant_correct_1024(ce_ctx* ctx, const float* B, int R, float* y, cudaStr
   if (ctx->P != P || m > P / 2) return fail(ctx, CE_ERR_ARG, "register circulant correction: P = 1024 only");
   const int pairs = (R + 1) / 2;
   const int chunk = ctx->circ_pairs;
-  const size_t shm = sizeof(float2) * std::max((size_t)kFastWarps * 32 * 33, (size_t)m * (kFastWarps + 1));
-  CE_CUDA_TRY(cudaFuncSetAttribute(circ1024_rowfwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-  CE_CUDA_TRY(cudaFuncSetAttribute(circ1024_col_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+  constexpr size_t shm = sizeof(float2) * kFastWarps * 32 * 33;   // holds the staged m x 9 elements too
+  static_assert(P / 2 * (kFastWarps + 1) <= kFastWarps * 32 * 33, "the column stage fits the transpose buffers");
+  CE_CUDA_TRY(set_max_smem(circ1024_rowfwd_kernel, shm));
+  CE_CUDA_TRY(set_max_smem(circ1024_col_kernel, shm));
   const size_t shm_r = sizeof(float2) * (size_t)kFastWarps * kLineBuf;
-  CE_CUDA_TRY(cudaFuncSetAttribute(reg_rowout_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_r));
+  CE_CUDA_TRY(set_max_smem(reg_rowout_kernel<1, true>, shm_r));
   for (int p0 = 0; p0 < pairs; p0 += chunk) {
     const int np = std::min(chunk, pairs - p0);
     float2* S = ctx->Xc;

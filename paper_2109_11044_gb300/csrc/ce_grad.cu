@@ -240,7 +240,7 @@ template <int RT>
 int launch_grad_window(const float* v, int m, Window win, int R, const float4* obs, int nobs, CovF cov, double* csum,
                        double* dsum, long long nW, int nsm, cudaStream_t s) {
   using T = GradTile<RT>;
-  CE_CUDA_TRY(cudaFuncSetAttribute(grad_window_kernel<RT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem));
+  CE_CUDA_TRY(set_max_smem(grad_window_kernel<RT>, T::smem));
   const int qb = (nobs + T::QT - 1) / T::QT;
   // slices of the window: two blocks per SM in turn, at least 64 nodes each
   const int splits = (int)std::max<long long>(1, std::min<long long>(2 * nsm / qb, nW / 64));
@@ -251,6 +251,7 @@ int launch_grad_window(const float* v, int m, Window win, int R, const float4* o
 // sum over sites i, j of dA_ij (a_i a_j / 2 - Ainv_ij / 2 - sum_r w_r,i B_r,j), for
 // dA = 2 K_oo / sigma, dK_oo / dtheta and I: acc[0..2].
 constexpr int GP_T = 32;
+constexpr int kGradMaxR = 128;   // realizations of one gradient call
 
 __global__ void __launch_bounds__(256) grad_pairs_kernel(const float* __restrict__ w, const float* __restrict__ B, int ldb,
                                                          int R, int nobs, const float4* __restrict__ obs,
@@ -403,7 +404,7 @@ extern "C" int ce_condsim_grad(ce_ctx* ctx, const float* z_dev, int R, uint64_t 
   ctx->err.clear();
   if (ctx->mode != CE_LOCAL) return fail(ctx, CE_ERR_STATE, "the gradient needs local Kriging (ce_krige_weights, CE_LOCAL)");
   if (!z_dev || !window || !out_dev || !grad_theta || !grad_z_dev || !loss) return fail(ctx, CE_ERR_ARG, "null pointer");
-  if (R < 1 || R > 128) return fail(ctx, CE_ERR_ARG, "the gradient takes 1 <= R <= 128");
+  if (R < 1 || R > kGradMaxR) return fail(ctx, CE_ERR_ARG, "the gradient takes 1 <= R <= 128");
   const Window win{window[0], window[1], window[2], window[3]};
   if (win.i0 < 0 || win.j0 < 0 || win.i1 > ctx->m || win.j1 > ctx->m || win.i0 >= win.i1 || win.j0 >= win.j1)
     return fail(ctx, CE_ERR_ARG, "window must be a non-empty sub-rectangle of the grid");
@@ -461,7 +462,7 @@ extern "C" int ce_condsim_grad(ce_ctx* ctx, const float* z_dev, int R, uint64_t 
   // 3. prediction matrix and log-likelihood
   {
     const size_t shm = sizeof(float) * 2 * (size_t)R * GP_T;
-    CE_CUDA_TRY(cudaFuncSetAttribute(grad_pairs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+    CE_CUDA_TRY(set_max_smem(grad_pairs_kernel, sizeof(float) * 2 * kGradMaxR * GP_T));
     dim3 g((n + GP_T - 1) / GP_T, (n + GP_T - 1) / GP_T);
     grad_pairs_kernel<<<g, 256, shm, s>>>(w, ctx->Bm, ctx->nobs_pad, R, n, ctx->obs, alpha, ctx->Ainv_hi, ctx->Ainv_lo,
                                           ctx->nobs_pad, cov, inv_sigma, acc + 2);

@@ -316,6 +316,9 @@ __device__ __forceinline__ double scaled_double(long long T, int e) {
   return T == 0 ? 0.0 : __longlong_as_double((long long)(bits | ((unsigned long long)T & 0x8000000000000000ull)));
 }
 
+// Dynamic shared memory of a panel block: its rows of the panel and of V.
+constexpr size_t panel_smem(int rows) { return sizeof(double) * 2 * (size_t)rows * (kW + 2); }
+
 constexpr uint32_t kUpdateSmem = kDigits * (kABlock + kBBlock) + 1024;
 
 // M -= V V^T on the 128 x 64 tile (I, J) of the lower triangle, the swept block's own rows
@@ -526,16 +529,16 @@ int spd_inverse_f64(ce_ctx* ctx, double* M, int n, cudaStream_t s, double* logde
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(sweep_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kUpdateSmem);
+    e = set_max_smem(sweep_update_kernel, kUpdateSmem);
   // panel rows per thread block: one block per SM until a block would hold more than kMaxRows
   // (the FP64 units of every SM take part; each block also factors the pivot)
   int rows = nsm > 0 ? (np + nsm - 1) / nsm : kMaxRows;
   rows = rows < 4 ? 4 : (rows > kMaxRows ? kMaxRows : rows);
   const unsigned gp = (unsigned)((np + rows - 1) / rows);
   const unsigned T = (unsigned)(np / 128);
-  const size_t shp = sizeof(double) * 2 * (size_t)rows * (kW + 2);
+  const size_t shp = panel_smem(rows);
   for (auto k : {panel_kernel<0>, panel_kernel<1>})
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shp);
+    if (e == cudaSuccess) e = set_max_smem(k, panel_smem(kMaxRows));
   for (int k0 = 0; e == cudaSuccess && k0 < n; k0 += kW) {
     panel_kernel<0><<<gp, 256, shp, s>>>(M, np, k0, rows, nullptr, Pa, V0, nullptr, nullptr, piv, ctx->dev_status);
     panel_kernel<1><<<gp, 256, shp, s>>>(M, np, k0, rows, Pa, Pb, V0, vd, ve, piv, ctx->dev_status);

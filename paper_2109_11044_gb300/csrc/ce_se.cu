@@ -508,7 +508,7 @@ extern "C" int ce_se_map(ce_ctx* ctx, float* se_exact_dev, float* se_approx_dev,
   }
   int st = CE_OK, parts = 0;
   {
-    const cudaError_t ea = cudaFuncSetAttribute(se_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem);
+    const cudaError_t ea = set_max_smem(se_gemm_kernel, kGemmSmem);
     if (ea != cudaSuccess) st = cuda_fail(ea, "standard errors", __FILE__, __LINE__);
   }
   for (long long g0 = 0; g0 < M && st == CE_OK; g0 += Mc) {

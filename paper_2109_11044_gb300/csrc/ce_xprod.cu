@@ -40,6 +40,7 @@ constexpr int kAPlanes = 5, kBPlanes = 4;   // digits of a matrix element, of an
 constexpr uint32_t kAPlane = 128 * 128; // bytes of one digit plane: 128 rows x 64 columns of bf16
 constexpr int kUnit = 4;                // chunks of 64 columns summed in tensor memory
 constexpr int kMaxRing = 8;             // digit planes of the matrix in flight
+constexpr uint32_t kXprodSmem = 226 * 1024;   // most dynamic shared memory of a block
 constexpr int kEpi = 8;                 // epilogue warps
 constexpr int kThreads = (kEpi + 2) * 32;
 
@@ -432,9 +433,9 @@ int launch_xprod(ce_ctx* ctx, const float* E, long long lde, int R, int n, const
   a.kparts = kp;
   a.items = mt * nb * kp;
   const uint32_t bbytes = 2u * kBPlanes * (uint32_t)np * 128u;
-  a.ring = std::min<int>(kMaxRing, (int)((226u * 1024u - 1024u - bbytes) / kAPlane));
+  a.ring = std::min<int>(kMaxRing, (int)((kXprodSmem - 1024u - bbytes) / kAPlane));
   const size_t smem = (size_t)bbytes + (size_t)a.ring * kAPlane + 1024;
-  CE_CUDA_TRY(cudaFuncSetAttribute(xprod_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  CE_CUDA_TRY(set_max_smem(xprod_kernel, kXprodSmem));
   digit_rows_kernel<kBPlanes><<<nb * np, 256, 0, s>>>(E, nullptr, lde, R, n, np, nc, planes, bscale);
   xprod_kernel<<<std::min(a.items, nsm), kThreads, smem, s>>>(a);
   CE_CUDA_TRY(cudaGetLastError());
