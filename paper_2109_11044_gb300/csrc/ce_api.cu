@@ -148,9 +148,11 @@ int ce_setup(ce_ctx** out, const ce_grid* grid, const ce_cov* cov, int max_growt
   ctx->nu = cov->nu;
   ctx->tau2 = cov->tau2;
   ctx->setup_stream = as_stream(stream);
-  ctx->dev_status = (int*)dalloc(ctx, 4 * sizeof(int));   // the status word, then the work-queue counter
+  // the status word, the work-queue counter, the set-up's own status word
+  ctx->dev_status = (int*)dalloc(ctx, 4 * sizeof(int));
   if (!ctx->dev_status) { delete ctx; return fail(nullptr, CE_ERR_OOM, "status word"); }
   ctx->queue = reinterpret_cast<unsigned*>(ctx->dev_status + 1);
+  ctx->setup_status = ctx->dev_status + 2;
   if (cudaMemset(ctx->dev_status, 0, 4 * sizeof(int)) != cudaSuccess) {
     ce_destroy(ctx);
     return fail(nullptr, CE_ERR_CUDA, "status word");

@@ -100,7 +100,8 @@ struct ce_ctx {
   cudaEvent_t ev_computed[2] = {nullptr, nullptr}, ev_copied[2] = {nullptr, nullptr};
   int async_slot = 0;
   float* zdev_tmp = nullptr;
-  int* dev_status = nullptr;    // device-side error word
+  int* dev_status = nullptr;    // device-side error word of the queued calls (ce_sync_status)
+  int* setup_status = nullptr;  // that of the inverse, which reports it itself (beside the error word)
   unsigned* queue = nullptr;    // work-queue counter of the tensor-core correction (beside the status word)
   unsigned wait_limit = 1u << 22;  // bound on the correction's accumulator waits (ce_set_wait_limit)
   cudaStream_t setup_stream = nullptr;

@@ -513,7 +513,7 @@ __global__ void __launch_bounds__(256) finish_inverse_kernel(double* __restrict_
 
 int spd_inverse_f64(ce_ctx* ctx, double* M, int n, cudaStream_t s, double* logdet) {
   const int np = (n + 127) / 128 * 128;
-  CE_CUDA_TRY(cudaMemsetAsync(ctx->dev_status, 0, sizeof(int), s));
+  CE_CUDA_TRY(cudaMemsetAsync(ctx->setup_status, 0, sizeof(int), s));
   // one block of work memory: two panels, half of V, the digits of V, the pivots, the exponents
   const size_t panel = sizeof(double) * (size_t)np * kW;
   const size_t dig = (size_t)np * kDigits * 128;   // 128 bytes per row and digit
@@ -540,14 +540,14 @@ int spd_inverse_f64(ce_ctx* ctx, double* M, int n, cudaStream_t s, double* logde
   for (auto k : {panel_kernel<0>, panel_kernel<1>})
     if (e == cudaSuccess) e = set_max_smem(k, panel_smem(kMaxRows));
   for (int k0 = 0; e == cudaSuccess && k0 < n; k0 += kW) {
-    panel_kernel<0><<<gp, 256, shp, s>>>(M, np, k0, rows, nullptr, Pa, V0, nullptr, nullptr, piv, ctx->dev_status);
-    panel_kernel<1><<<gp, 256, shp, s>>>(M, np, k0, rows, Pa, Pb, V0, vd, ve, piv, ctx->dev_status);
-    sweep_update_kernel<<<T * (T + 1), 288, kUpdateSmem, s>>>(M, np, k0, Pb, vd, ve, ctx->dev_status);
+    panel_kernel<0><<<gp, 256, shp, s>>>(M, np, k0, rows, nullptr, Pa, V0, nullptr, nullptr, piv, ctx->setup_status);
+    panel_kernel<1><<<gp, 256, shp, s>>>(M, np, k0, rows, Pa, Pb, V0, vd, ve, piv, ctx->setup_status);
+    sweep_update_kernel<<<T * (T + 1), 288, kUpdateSmem, s>>>(M, np, k0, Pb, vd, ve, ctx->setup_status);
   }
   if (e == cudaSuccess) e = cudaGetLastError();
   int st = 0;
   std::vector<double> hp(n);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&st, ctx->dev_status, sizeof(int), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&st, ctx->setup_status, sizeof(int), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(hp.data(), piv, sizeof(double) * n, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   dfree(ctx, buf);

@@ -1,0 +1,53 @@
+"""Statuses that kernels record: a set-up neither hides one nor leaves one behind.  The expired
+waits are made by a wait limit of zero rounds (ce_set_wait_limit), which ends a launch with
+CE_ERR_TIMEOUT and nothing else."""
+import pytest
+
+import workloads
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ce():
+    from paper_2109_11044_gb300.build import build
+    build()
+    import paper_2109_11044_gb300 as mod
+    mod.load_library()
+    return mod
+
+
+def _sited(ce, n, prec, m=64):
+    wl = workloads.workload("plain64").scaled(m=m, n=n)
+    sites = workloads.make_sites(wl)
+    z = torch.tensor(workloads.make_data(wl, sites), dtype=torch.float32, device="cuda")
+    return ce.Context.from_workload(wl).krige_weights(sites, "local", np_=2, prec=prec), sites, z
+
+
+def _expires(ce, call):
+    with pytest.raises(ce.CEError) as e:
+        call()
+    assert e.value.status == ce.CE_ERR_TIMEOUT
+
+
+def test_a_set_up_keeps_a_pending_status(ce):
+    ctx, sites, z = _sited(ce, 200, "f16x3")
+    ctx.set_wait_limit(0)
+    ctx.condsim(z, 4, 3)
+    torch.cuda.synchronize()
+    ctx.set_wait_limit(1 << 22)
+    ctx.krige_weights(sites, "local", np_=2, prec="f16x3")
+    _expires(ce, ctx.sync)
+
+
+def test_a_refused_set_up_leaves_no_status(ce):
+    wl = workloads.workload("plain64").scaled(n=70, tau2=0.0)
+    sites = workloads.make_sites(wl)
+    sites[69] = sites[3]
+    ctx = ce.Context.from_workload(wl)
+    with pytest.raises(ce.CEError) as e:
+        ctx.krige_weights(sites, "local", np_=2)
+    assert e.value.status == ce.CE_ERR_NOT_SPD
+    ctx.unconditional(2, 1)
+    ctx.sync()
