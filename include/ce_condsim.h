@@ -173,18 +173,19 @@ int ce_set_precision(ce_ctx* ctx, int prec);
 enum ce_solve_form { CE_SOLVE_FP32 = 0, CE_SOLVE_TENSOR = 1 };
 int ce_set_solve_form(ce_ctx* ctx, int form);
 
-/* Bound on each wait of the tensor-core correction's epilogue for an accumulator
- * (no counterpart in the paper): the number of mbarrier try_wait rounds (each of
- * which suspends the waiting thread for at most 2 us, less when the accumulator
- * becomes ready) before the wait gives up, records CE_ERR_TIMEOUT, and the launch aborts; the launch then
- * lets its bulk copies and tensor-core work finish, frees its tensor memory and
- * returns, and ce_sync_status reports CE_ERR_TIMEOUT (once: the status word is
- * cleared as it is read).  The output of such a call is invalid.  Default 2^22
- * rounds (at most about 8 s); 0 makes every such wait give up at once, which exercises the
- * abort path without a fault.  Applies to later calls on this context, and to the
- * shared correction launch of a batch (ce_condsim_batch, ce_batch_create) whose
- * first joined event, in the caller's order, it is; that launch reports its status
- * on the same context. */
+/* Bound on each wait of an epilogue for a tensor-memory accumulator, in the tensor-core
+ * correction and in the set-up's matrix updates (no counterpart in the paper): the
+ * number of mbarrier try_wait rounds (each of which suspends the waiting thread for at
+ * most 2 us, less when the accumulator becomes ready) before the wait gives up, records
+ * CE_ERR_TIMEOUT, and the launch aborts; the launch then lets its bulk copies and
+ * tensor-core work finish, frees its tensor memory and returns, and ce_sync_status
+ * reports CE_ERR_TIMEOUT (once: the status word is cleared as it is read);
+ * ce_krige_weights returns its own CE_ERR_TIMEOUT.  The output of such a call is
+ * invalid.  Default 2^22 rounds (at most about 8 s); 0 makes every such wait give up at
+ * once, which exercises the abort path without a fault.  Applies to later calls on this
+ * context, and to the shared correction launch of a batch (ce_condsim_batch,
+ * ce_batch_create) whose first joined event, in the caller's order, it is; that launch
+ * reports its status on the same context. */
 int ce_set_wait_limit(ce_ctx* ctx, unsigned iterations);
 
 /* How the Kriging correction K_gN B (step 5) is formed in NN mode.

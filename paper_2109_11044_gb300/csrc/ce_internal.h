@@ -103,7 +103,7 @@ struct ce_ctx {
   int* dev_status = nullptr;    // device-side error word of the queued calls (ce_sync_status)
   int* setup_status = nullptr;  // that of the inverse, which reports it itself (beside the error word)
   unsigned* queue = nullptr;    // work-queue counter of the tensor-core correction (beside the status word)
-  unsigned wait_limit = 1u << 22;  // bound on the correction's accumulator waits (ce_set_wait_limit)
+  unsigned wait_limit = 1u << 22;  // bound on the epilogues' accumulator waits (ce_set_wait_limit)
   cudaStream_t setup_stream = nullptr;
   size_t device_bytes = 0;
   std::unordered_map<void*, size_t> allocs;

@@ -102,7 +102,7 @@ __device__ __forceinline__ void factor32(double (&a)[4], double (&rowb)[2][kH], 
           // positive, normal and finite by its bits (an FP64 compare takes 64 cycles of this chain)
           const long long b = __double_as_longlong(p);
           if (b < 0x0010000000000000ll || b >= 0x7ff0000000000000ll) {   // not positive definite
-            atomicExch(status, CE_ERR_NOT_SPD);
+            atomicMax(status, CE_ERR_NOT_SPD);   // an expired wait, which can lead to this, stays the reported one
             p = 1.0;
           }
           rpb[kr & 1] = recip_pos(p);
@@ -322,10 +322,12 @@ constexpr size_t panel_smem(int rows) { return sizeof(double) * 2 * (size_t)rows
 constexpr uint32_t kUpdateSmem = kDigits * (kABlock + kBBlock) + 1024;
 
 // M -= V V^T on the 128 x 64 tile (I, J) of the lower triangle, the swept block's own rows
-// and columns taken from the panel P.  Warps 0-7: epilogue; warp 8: copies and MMA.
+// and columns taken from the panel P.  Warps 0-7: epilogue, which waits for the products at most
+// epi_wait rounds; warp 8: copies and MMA, which has seen both finish (within its own bound)
+// before the block frees its tensor memory and exits, also when the epilogue has given up.
 __global__ void __launch_bounds__(288) sweep_update_kernel(double* __restrict__ M, int np, int k0, const double* __restrict__ P,
                                                            const uint8_t* __restrict__ dig, const int* __restrict__ dexp,
-                                                           int* __restrict__ status) {
+                                                           uint32_t epi_wait, int* __restrict__ status) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   __shared__ __align__(8) uint64_t bars[3];   // A digit 0 and B; A digits 1-6; products done
@@ -359,9 +361,9 @@ __global__ void __launch_bounds__(288) sweep_update_kernel(double* __restrict__ 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
-  auto wait = [&](int b) {
+  auto wait = [&](int b, uint32_t limit) {
     bool done = false;
-    for (uint32_t it = 0; it < kWaitLimit && !done; ++it) done = mbar_try_for(smem_u32(&bars[b]), 0u, 2000u);
+    for (uint32_t it = 0; it < limit && !done; ++it) done = mbar_try_for(smem_u32(&bars[b]), 0u, 2000u);
     return done;
   };
   if (warp == 8) {
@@ -377,12 +379,12 @@ __global__ void __launch_bounds__(288) sweep_update_kernel(double* __restrict__ 
           bulk_g2s(base + (uint32_t)t * kABlock + (uint32_t)h * kBBlock, va + (size_t)(h * kDigits + t) * kBBlock, kBBlock,
                    smem_u32(&bars[t ? 1 : 0]));
       const uint32_t ibase = (1u << 4) | ((uint32_t)(128 >> 4) << 24);
-      bool ok = wait(0);
+      bool ok = wait(0, kWaitLimit);
       tc_fence_after();
 #pragma unroll 1
       for (int t = 0; t < kDigits; ++t) {
         if (t == 1) {   // waited for in any case: no copy is in flight when the block exits
-          ok = wait(1) && ok;
+          ok = wait(1, kWaitLimit) && ok;
           tc_fence_after();
         }
         if (!ok) continue;
@@ -400,7 +402,8 @@ __global__ void __launch_bounds__(288) sweep_update_kernel(double* __restrict__ 
         }
       }
       mma_commit(smem_u32(&bars[2]));
-      if (!ok) atomicExch(status, CE_ERR_TIMEOUT);
+      ok = wait(2, kWaitLimit) && ok;
+      if (!ok) atomicMax(status, CE_ERR_TIMEOUT);
     }
     __syncwarp();
   } else {
@@ -419,9 +422,9 @@ __global__ void __launch_bounds__(288) sweep_update_kernel(double* __restrict__ 
     };
     read8(0);
     const int we = dexp[r];
-    const bool ok = __all_sync(0xffffffffu, wait(2));
+    const bool ok = __all_sync(0xffffffffu, wait(2, epi_wait));
     tc_fence_after();
-    if (!ok && lane == 0) atomicExch(status, CE_ERR_TIMEOUT);
+    if (!ok && lane == 0) atomicMax(status, CE_ERR_TIMEOUT);
     if (ok && lower) {
 #pragma unroll 1
       for (int c = 0; c < 32; c += 8) {
@@ -542,7 +545,7 @@ int spd_inverse_f64(ce_ctx* ctx, double* M, int n, cudaStream_t s, double* logde
   for (int k0 = 0; e == cudaSuccess && k0 < n; k0 += kW) {
     panel_kernel<0><<<gp, 256, shp, s>>>(M, np, k0, rows, nullptr, Pa, V0, nullptr, nullptr, piv, ctx->setup_status);
     panel_kernel<1><<<gp, 256, shp, s>>>(M, np, k0, rows, Pa, Pb, V0, vd, ve, piv, ctx->setup_status);
-    sweep_update_kernel<<<T * (T + 1), 288, kUpdateSmem, s>>>(M, np, k0, Pb, vd, ve, ctx->setup_status);
+    sweep_update_kernel<<<T * (T + 1), 288, kUpdateSmem, s>>>(M, np, k0, Pb, vd, ve, ctx->wait_limit, ctx->setup_status);
   }
   if (e == cudaSuccess) e = cudaGetLastError();
   int st = 0;

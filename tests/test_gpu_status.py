@@ -31,6 +31,18 @@ def _expires(ce, call):
     assert e.value.status == ce.CE_ERR_TIMEOUT
 
 
+@pytest.mark.parametrize("n", [60, 200, 700])
+def test_expired_wait_in_the_set_up(ce, n):
+    ctx, sites, z = _sited(ce, n, "fp32")
+    want, logdet = ctx.condsim(z, 3, 7), ctx.info()["logdet"]
+    ctx.set_wait_limit(0)
+    _expires(ce, lambda: ctx.krige_weights(sites, "local", np_=2))
+    ctx.set_wait_limit(1 << 22)
+    ctx.sync()   # nothing left behind
+    ctx.krige_weights(sites, "local", np_=2)
+    assert ctx.info()["logdet"] == logdet and torch.equal(ctx.condsim(z, 3, 7), want)
+
+
 def test_a_set_up_keeps_a_pending_status(ce):
     ctx, sites, z = _sited(ce, 200, "f16x3")
     ctx.set_wait_limit(0)
