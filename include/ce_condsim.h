@@ -174,18 +174,20 @@ enum ce_solve_form { CE_SOLVE_FP32 = 0, CE_SOLVE_TENSOR = 1 };
 int ce_set_solve_form(ce_ctx* ctx, int form);
 
 /* Bound on each wait of an epilogue for a tensor-memory accumulator, in the tensor-core
- * correction and in the set-up's matrix updates (no counterpart in the paper): the
- * number of mbarrier try_wait rounds (each of which suspends the waiting thread for at
- * most 2 us, less when the accumulator becomes ready) before the wait gives up, records
- * CE_ERR_TIMEOUT, and the launch aborts; the launch then lets its bulk copies and
- * tensor-core work finish, frees its tensor memory and returns, and ce_sync_status
- * reports CE_ERR_TIMEOUT (once: the status word is cleared as it is read);
- * ce_krige_weights returns its own CE_ERR_TIMEOUT.  The output of such a call is
- * invalid.  Default 2^22 rounds (at most about 8 s); 0 makes every such wait give up at
- * once, which exercises the abort path without a fault.  Applies to later calls on this
- * context, and to the shared correction launch of a batch (ce_condsim_batch,
- * ce_batch_create) whose first joined event, in the caller's order, it is; that launch
- * reports its status on the same context. */
+ * correction, in the products from 8-bit digits (ce_set_solve_form, ce_se_map) and in
+ * the set-up's matrix updates (no counterpart in the paper): the number of mbarrier
+ * try_wait rounds (each of which suspends the waiting thread for at most 2 us, less when
+ * the accumulator becomes ready) before the wait gives up, records CE_ERR_TIMEOUT, and
+ * the launch aborts; the launch then lets its bulk copies and tensor-core work finish,
+ * frees its tensor memory and returns, and ce_sync_status or the next call that
+ * synchronises and reads the status (ce_condsim_host, ce_host_wait, ce_condsim_grad,
+ * ce_se_map) reports CE_ERR_TIMEOUT (once: the status word is cleared as it is read);
+ * ce_krige_weights returns its own CE_ERR_TIMEOUT.  The output of such a call is invalid.
+ * Default 2^22 rounds (at most about 8 s); 0 makes every such wait give up at once, which
+ * exercises the abort path without a fault.  Applies to later calls on this context, and
+ * to the shared correction launch of a batch (ce_condsim_batch, ce_batch_create) whose
+ * first joined event, in the caller's order, it is; that launch reports its status on the
+ * same context. */
 int ce_set_wait_limit(ce_ctx* ctx, unsigned iterations);
 
 /* How the Kriging correction K_gN B (step 5) is formed in NN mode.
@@ -248,7 +250,9 @@ int ce_set_box_joint(ce_ctx* ctx, int on, int* n_boxes);
  * CE_ERR_STATE while a trend is set.  Cost in local mode: two products of
  * M x n by n x n (M grid nodes; 177 ms in all at 512 x 512, n = 2000, 36 window
  * nodes).  Allocates its work buffers (about 300 MB
- * at most, plus n x n pairs and an m x (2m - 1) table) and synchronises `stream`. */
+ * at most; se_approx in local mode: 18 n^2 bytes more for Q's pair and digits, and an
+ * m x (2m - 1) table), synchronises `stream` and returns a status that a kernel
+ * recorded, as ce_condsim_host does. */
 int ce_se_map(ce_ctx* ctx, float* se_exact_dev, float* se_approx_dev, void* stream);
 
 /* Ensemble moments at every grid node (the ensemble mean estimate and its
@@ -297,7 +301,8 @@ int ce_condsim_prepare(ce_ctx* ctx, int R);
 /* ce_condsim with host buffers: copies z (n floats) to the device, runs
  * ce_condsim into a context-owned buffer and copies R x m x m floats back
  * to out_host.  Pinned host memory gives full copy bandwidth.  Returns after
- * the copy-back has completed. */
+ * the copy-back has completed, with the status that a kernel recorded, if any (as
+ * ce_sync_status does: an expired wait of this call, or of calls queued before it). */
 int ce_condsim_host(ce_ctx* ctx, const float* z_host, int R, uint64_t seed, uint64_t r_offset,
                     float* out_host, void* stream);
 
@@ -407,7 +412,8 @@ int ce_unconditional_static(ce_ctx* ctx, int R, uint64_t seed, uint64_t r_offset
  * dL/d(sigma, range, tau^2); grad_z_dev (device float, n) receives dL/dz in the
  * caller's site order; *loss receives L.  1 <= R <= 128.  The first call sets
  * up the derivatives of the spectral weights and of the off-grid weights (FP64).
- * Synchronises the stream.
+ * Synchronises the stream; a status that a kernel recorded is returned, as by
+ * ce_condsim_host, and grad_theta and *loss are not written then.
  * ------------------------------------------------------------------------- */
 int ce_condsim_grad(ce_ctx* ctx, const float* z_dev, int R, uint64_t seed, uint64_t r_offset, const int* window,
                     float* out_dev, double* grad_theta, float* grad_z_dev, double* loss, void* stream);

@@ -209,8 +209,9 @@ class Context:
         _check(load_library().ce_set_solve_form(self._ctx, SOLVE_FORMS[form]), self._ctx)
 
     def set_wait_limit(self, iterations: int):
-        """ce_set_wait_limit: bound (try_wait rounds) on the tensor-core correction's
-        accumulator waits; 0 makes them give up at once (the call reports CE_ERR_TIMEOUT)."""
+        """ce_set_wait_limit: bound (try_wait rounds) on the epilogues' accumulator waits (the
+        tensor-core correction, the digit products, the set-up); 0 makes them give up at once (the
+        call, or sync() after it, reports CE_ERR_TIMEOUT)."""
         _check(load_library().ce_set_wait_limit(self._ctx, int(iterations)), self._ctx)
         return self
 

@@ -107,6 +107,18 @@ void data_to_internal(ce_ctx* ctx, const float* z, cudaStream_t s) {
 
 namespace ce {
 
+int sync_stream_status(ce_ctx* ctx, cudaStream_t s) {
+  int st = 0;
+  CE_CUDA_TRY(cudaMemcpyAsync(&st, ctx->dev_status, sizeof(int), cudaMemcpyDeviceToHost, s));
+  CE_CUDA_TRY(cudaStreamSynchronize(s));
+  if (!st) return CE_OK;
+  // reported once: the next calls start from a clear status word
+  CE_CUDA_TRY(cudaMemsetAsync(ctx->dev_status, 0, sizeof(int), s));
+  CE_CUDA_TRY(cudaStreamSynchronize(s));
+  return fail(ctx, st, "a kernel reported status " + std::to_string(st) +
+                           (st == CE_ERR_TIMEOUT ? " (a bounded device wait gave up; the call's output is invalid)" : ""));
+}
+
 int condsim_front(ce_ctx* ctx, const float* z, int R, uint64_t seed, uint64_t r_offset, float* out, cudaStream_t s) {
   int st = check_call(ctx, R, r_offset);
   if (st) return st;
@@ -356,8 +368,7 @@ int ce_condsim_host(ce_ctx* ctx, const float* z_host, int R, uint64_t seed, uint
   CE_CUDA_TRY(cudaMemcpyAsync(ctx->zdev_tmp, z_host, sizeof(float) * ctx->n, cudaMemcpyHostToDevice, s));
   if ((st = ce_condsim(ctx, ctx->zdev_tmp, R, seed, r_offset, ctx->host_out, stream))) return st;
   CE_CUDA_TRY(cudaMemcpyAsync(out_host, ctx->host_out, bytes, cudaMemcpyDeviceToHost, s));
-  CE_CUDA_TRY(cudaStreamSynchronize(s));
-  return CE_OK;
+  return sync_stream_status(ctx, s);
 }
 
 int ce_condsim_host_async(ce_ctx* ctx, const float* z_host, int R, uint64_t seed, uint64_t r_offset, float* out_host,
@@ -521,15 +532,7 @@ int ce_copy_array(const ce_ctx* cctx, int which, void* dst, size_t bytes) {
 int ce_sync_status(ce_ctx* ctx) {
   if (!ctx) return fail(nullptr, CE_ERR_ARG, "null context");
   CE_CUDA_TRY(cudaDeviceSynchronize());
-  int st = 0;
-  CE_CUDA_TRY(cudaMemcpy(&st, ctx->dev_status, sizeof(int), cudaMemcpyDeviceToHost));
-  if (st) {
-    // reported once: the next calls start from a clear status word
-    CE_CUDA_TRY(cudaMemset(ctx->dev_status, 0, sizeof(int)));
-    return fail(ctx, st, "a kernel reported status " + std::to_string(st) +
-                             (st == CE_ERR_TIMEOUT ? " (a bounded device wait gave up; the call's output is invalid)" : ""));
-  }
-  return CE_OK;
+  return sync_stream_status(ctx, nullptr);
 }
 
 const char* ce_last_error(const ce_ctx* ctx) {

@@ -485,8 +485,9 @@ extern "C" int ce_condsim_grad(ce_ctx* ctx, const float* z_dev, int R, uint64_t 
   CE_CUDA_TRY(cudaMemcpyAsync(h_acc, acc, sizeof(h_acc), cudaMemcpyDeviceToHost, s));
   CE_CUDA_TRY(cudaMemcpyAsync(h_alpha.data(), alpha, sizeof(float) * n, cudaMemcpyDeviceToHost, s));
   CE_CUDA_TRY(cudaMemcpyAsync(h_z.data(), ctx->zint, sizeof(float) * n, cudaMemcpyDeviceToHost, s));
-  CE_CUDA_TRY(cudaStreamSynchronize(s));
+  st = sync_stream_status(ctx, s);   // an expired wait left incomplete sums
   dfree(ctx, acc);
+  if (st) return st;
   // acc: [0,1] correction (sigma, theta); [2,3,4] pairs (sigma, theta, tau2);
   //      [5,6,7] off-grid (sigma, theta, tau2); [8,9] fields (theta, sigma); [10] sum of squares
   grad_theta[0] = h_acc[0] + h_acc[2] + h_acc[5] + h_acc[9];

@@ -129,6 +129,8 @@ int fail(ce_ctx* ctx, int status, const std::string& msg);
 void* dalloc(ce_ctx* ctx, size_t bytes);   // tracked cudaMalloc, nullptr on failure
 void dfree(ce_ctx* ctx, void* p);
 
+// ce_api.cu: synchronises s, then returns (and clears) the status that a kernel recorded
+int sync_stream_status(ce_ctx* ctx, cudaStream_t s);
 // ce_api.cu: allocate the per-call work buffers of R realizations ahead of time
 int ensure_fft_buffer(ce_ctx* ctx, int R);
 int ensure_bsplit(ce_ctx* ctx, int R);

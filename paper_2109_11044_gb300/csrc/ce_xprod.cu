@@ -130,6 +130,7 @@ struct XArgs {
   const float* bscale;
   float2* part;          // kparts x R x n pairs
   int n, R, npad, nchunks, nblocks, kparts, cpp, items, ring;
+  uint32_t epi_wait;     // bound on the epilogue's waits for an accumulator (try_wait rounds)
   int* status;
 };
 
@@ -312,7 +313,7 @@ __global__ void __launch_bounds__(kThreads) xprod_kernel(const __grid_constant__
 #pragma unroll
       for (int j = 0; j < 64; ++j) hi[j] = lo[j] = 0.f;
       for (int u = 0; u < units; ++u, ++unit) {
-        const bool got = mbar_wait(smem_u32(&acc_full), unit & 1u, &abort_flag);
+        const bool got = mbar_wait(smem_u32(&acc_full), unit & 1u, &abort_flag, p.epi_wait);
         if (!__all_sync(0xffffffffu, got)) {
           abort_flag = 1;
           if (lane == 0) atomicExch(p.status, CE_ERR_TIMEOUT);
@@ -413,6 +414,7 @@ int launch_xprod(ce_ctx* ctx, const float* E, long long lde, int R, int n, const
   a.npad = np;
   a.nchunks = nc;
   a.nblocks = nb;
+  a.epi_wait = ctx->wait_limit;
   a.status = ctx->dev_status;
   int nsm = 0, dev = 0;
   CE_CUDA_TRY(cudaGetDevice(&dev));

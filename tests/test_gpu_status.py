@@ -1,6 +1,7 @@
-"""Statuses that kernels record: a set-up neither hides one nor leaves one behind.  The expired
-waits are made by a wait limit of zero rounds (ce_set_wait_limit), which ends a launch with
-CE_ERR_TIMEOUT and nothing else."""
+"""Statuses that kernels record: a call that synchronises reports them itself, a set-up neither
+hides nor leaves one behind.  The expired waits are made by a wait limit of zero rounds
+(ce_set_wait_limit), which ends a launch with CE_ERR_TIMEOUT and nothing else."""
+import numpy as np
 import pytest
 
 import workloads
@@ -29,6 +30,49 @@ def _expires(ce, call):
     with pytest.raises(ce.CEError) as e:
         call()
     assert e.value.status == ce.CE_ERR_TIMEOUT
+
+
+@pytest.mark.parametrize("n,prec", [(200, "f16x3"), (1800, "fp32")])
+def test_synchronous_calls_report_an_expired_wait(ce, n, prec):
+    ctx, _, z = _sited(ce, n, prec)
+    zh, out = z.cpu().pin_memory(), torch.empty((4, 64, 64), pin_memory=True)
+    win = (8, 40, 8, 40)
+    grad = ctx.condsim_grad(z, 4, 3, win)
+    host = ctx.condsim_host(zh, 4, 3, out_host=out).clone()
+    ctx.set_wait_limit(0)
+    _expires(ce, lambda: ctx.condsim_grad(z, 4, 3, win))
+    _expires(ce, lambda: ctx.condsim_host(zh, 4, 3, out_host=out))
+    ctx.sync()   # each was reported once
+    ctx.set_wait_limit(1 << 22)
+    again = ctx.condsim_grad(z, 4, 3, win)
+    assert torch.equal(again[0], grad[0]) and np.allclose(again[1], grad[1], rtol=1e-5) and np.isclose(again[3], grad[3], rtol=1e-6)
+    assert torch.equal(ctx.condsim_host(zh, 4, 3, out_host=out), host)
+    ctx.sync()
+
+
+@pytest.mark.parametrize("n", [60, 300])
+def test_standard_errors_report_an_expired_wait(ce, n):
+    ctx, _, _ = _sited(ce, n, "fp32")
+    exact, approx = ctx.se_map()
+    ctx.set_wait_limit(0)
+    _expires(ce, ctx.se_map)
+    ctx.sync()
+    ctx.set_wait_limit(1 << 22)
+    again = ctx.se_map()
+    assert torch.equal(again[0], exact) and torch.equal(again[1], approx)
+
+
+@pytest.mark.parametrize("R", [1, 16, 130])
+def test_expired_wait_in_the_digit_solve(ce, R):
+    ctx, _, _ = _sited(ce, 1800, "fp32")
+    E = torch.randn((R, 1800), generator=torch.Generator().manual_seed(R)).cuda()
+    want = ctx.solve(E)
+    ctx.set_wait_limit(0)
+    ctx.solve(E)
+    _expires(ce, ctx.sync)
+    ctx.set_wait_limit(1 << 22)
+    assert torch.equal(ctx.solve(E), want)
+    ctx.sync()
 
 
 @pytest.mark.parametrize("n", [60, 200, 700])
