@@ -174,12 +174,19 @@ int launch_solve(ce_ctx* ctx, const float* E, int R, float* B, int ldb, cudaStre
 // ce_xprod.cu: E A^-1 on the tensor cores from 8-bit digits.  The digit planes of the n x n
 // pair hi + lo (row stride ld), in a buffer of xprod_matrix_bytes(n); those of R rows of E
 // take xprod_rows_bytes(n, R).  launch_xprod writes *kparts <= max_parts partial (sum,
-// compensation) pairs per output to part (kparts x R x n); E's rows of stride lde.
+// compensation) pairs per output to part (kparts x R x n); E's rows of stride lde.  Given the
+// pair, rows whose values span too many binades for E's digits take its FP32 product, whose
+// kSolveKSplit pairs go to part: *scale receives R device values, negative for such a row.
+struct XprodPair {
+  const float *hi, *lo;   // row stride ld, a multiple of 128; E's rows then have stride n
+  int ld;
+  int chain;              // products summed per compensated step, 2 or 4
+};
 size_t xprod_matrix_bytes(int n);
 size_t xprod_rows_bytes(int n, int R);
 void launch_xprod_matrix(const float* hi, const float* lo, int ld, int n, void* buf, cudaStream_t s);
-int launch_xprod(ce_ctx* ctx, const float* E, long long lde, int R, int n, const void* matrix, void* rows,
-                 float* part, int max_parts, int* kparts, cudaStream_t s);
+int launch_xprod(ce_ctx* ctx, const float* E, long long lde, int R, int n, const void* matrix, const XprodPair* pair,
+                 void* rows, float* part, int max_parts, int* kparts, const float** scale, cudaStream_t s);
 // From this many rows on the solve takes the tensor-core digits.
 constexpr int kXprodMin = 1800;
 // The context's solve form is the tensor-core one.

@@ -526,7 +526,7 @@ extern "C" int ce_se_map(ce_ctx* ctx, float* se_exact_dev, float* se_approx_dev,
       ctx->launches += 1;
     }
     if (need_u) {
-      st = launch_xprod(ctx, Wc, n, rows, n, qdig, rowdig, reinterpret_cast<float*>(Tc), 1, &parts, s);   // Q w_g
+      st = launch_xprod(ctx, Wc, n, rows, n, qdig, nullptr, rowdig, reinterpret_cast<float*>(Tc), 1, &parts, nullptr, s);   // Q w_g
       if (st) break;
       auto dot = ctx->np == 1 ? se_dot_kernel<1, 2>
                               : (ctx->np == 2 ? se_dot_kernel<1, 4> : (ctx->np == 3 ? se_dot_kernel<1, 6> : se_dot_kernel<1, 8>));

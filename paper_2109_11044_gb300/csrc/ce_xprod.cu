@@ -10,6 +10,9 @@
 // columns and three products: below 2^24 units), the rest together in a fourth, whose
 // rounding lies near 2^-40.  After at most 256 columns the accumulators join a float pair
 // (TwoSum of the first two, the others with the errors in the low part).
+// Rows of E whose values span too many binades for that (kWideRatio: a bad station, a sparse or
+// decaying right-hand side) take the FP32 products of the pair instead, tile by tile in the same
+// kernel once the digits are done: a launch of its own for them cost every call 6.5 us.
 // The matrix needs its 40 bits: the residuals of real data are smooth, A^-1 E cancels, and
 // the correction K_go B amplifies what is left.  At n = 10000 (condition 10^4) a matrix cut
 // at 2^-32 leaves 4e-4 in the draw, at 2^-40 8e-7; the FP32 CUDA-core form (compensated sums,
@@ -31,6 +34,7 @@
 
 #include "ce_common.cuh"
 #include "ce_internal.h"
+#include "ce_solve_tile.cuh"
 #include "ce_tc.cuh"
 
 namespace ce {
@@ -42,7 +46,9 @@ constexpr int kUnit = 4;                // chunks of 64 columns summed in tensor
 constexpr int kMaxRing = 8;             // digit planes of the matrix in flight
 constexpr uint32_t kXprodSmem = 226 * 1024;   // most dynamic shared memory of a block
 constexpr int kEpi = 8;                 // epilogue warps
-constexpr int kThreads = (kEpi + 2) * 32;
+// Loader, MMA and epilogue; with the FP32 products of the wide rows (CHAIN > 0) two warps more, so
+// that these have three groups of 128 threads.
+__host__ __device__ constexpr int xprod_threads(int chain) { return chain ? (kEpi + 4) * 32 : (kEpi + 2) * 32; }
 
 // The digits of f, |f| < 1 (plus the low part g, |g| <= 2^-24 |f|), as bf16 bits in the
 // upper halves of d: each is the remainder rounded to a multiple of 2^-(7 + 8 t).
@@ -66,24 +72,40 @@ __device__ __forceinline__ uint32_t piece(int r, int kg) { return (uint32_t)r * 
 // normal number (above 2^127 the leading digit reaches 256, which bf16 holds too).
 __device__ __forceinline__ int exp_above(unsigned mx) { return max(-120, min(127, (int)(mx >> 23) - 126)); }
 
+// A row of E is wide where some kWideSites neighbouring sites (columns) all lie more than
+// kWideRatio below its largest element, or that lies outside [2^-100, 2^100).  E's digits leave
+// 2^-32.8 (RMS) of the row's largest element in every element, the FP32 products' roundings 2^-25.5
+// of each term: they meet where a neighbourhood lies 2^-7 below (n = 2000, one element of a normal
+// row raised to f: error of B half the domain away 2.6e-8 at f = 32, 4.1e-8 at 128, 7.9e-8 at
+// 256, 2e-6 at 10^4; by FP32 products 4e-8 at all).
+constexpr int kWideSites = 32;
+constexpr float kWideRatio = 128.f;
+
 // kPlanes digit planes of rows [0, rows) of v (row stride ldv, n columns; lo: the low parts or
 // null), one block per row.  Row r goes to row r % tile of tile r / tile: planes of tile x
 // 128 bytes, kPlanes of them per chunk of 64 columns, nchunks chunks per tile.  Rows past
 // `rows` and columns past n are zeros.  scale[r]: the power of two to multiply back by
-// (NaN where the row is not finite).
+// (NaN where the row is not finite), negative for a wide row of E.
 template <int kPlanes>
 __global__ void __launch_bounds__(256) digit_rows_kernel(const float* __restrict__ v, const float* __restrict__ lo, long long ldv,
                                                          int rows, int n, int tile, int nchunks, uint8_t* __restrict__ out,
                                                          float* __restrict__ scale) {
+  constexpr bool kRange = kPlanes == kBPlanes;
   __shared__ unsigned wmax[8];
   const int r = blockIdx.x;
   const bool live = r < rows;
   const float* __restrict__ src = v + (long long)(live ? r : 0) * ldv;
   const float* __restrict__ srl = lo ? lo + (long long)(live ? r : 0) * ldv : nullptr;
-  unsigned mx = 0;
-  if (live)
+  unsigned mx = 0, last = 0;   // last: of the row's last kWideSites columns, which may not be a group below
+  if (live) {
+    if (kRange && threadIdx.x < kWideSites && threadIdx.x < n)
+      last = __float_as_uint(src[max(n - kWideSites, 0) + threadIdx.x]) & 0x7fffffffu;
     for (int c = threadIdx.x; c < n; c += 256) mx = max(mx, __float_as_uint(src[c]) & 0x7fffffffu);
-  for (int o = 16; o; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  }
+  for (int o = 16; o; o >>= 1) {
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (kRange) last = max(last, __shfl_xor_sync(0xffffffffu, last, o));
+  }
   if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = mx;
   __syncthreads();
 #pragma unroll
@@ -91,17 +113,21 @@ __global__ void __launch_bounds__(256) digit_rows_kernel(const float* __restrict
   const bool finite = mx < 0x7f800000u;
   const int e = exp_above(mx);
   const float down = e == 127 ? 0x1p-127f : __uint_as_float((uint32_t)(127 - e) << 23);
-  if (threadIdx.x == 0) scale[r] = finite ? __uint_as_float((uint32_t)(127 + e) << 23) : __uint_as_float(0x7fc00000u);
   uint8_t* __restrict__ dst = out + (size_t)(r / tile) * nchunks * kPlanes * (size_t)tile * 128u;
   const int rr = r % tile;
+  const float top = __uint_as_float(mx) * down;   // (1/2, 1] wherever the row is not wide for its range alone
+  bool below = threadIdx.x < 32 && __uint_as_float(last) * down * kWideRatio < top;
   for (int p = threadIdx.x; p < nchunks * 8; p += 256) {   // pieces of eight columns
     uint32_t w[kPlanes][4];
+    float group = 0.f;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int c = p * 8 + j;
       const bool in = live && finite && c < n;
       uint32_t d[kPlanes];
-      digits<kPlanes>(in ? src[c] * down : 0.f, in && srl ? srl[c] * down : 0.f, d);
+      const float x = in ? src[c] * down : 0.f;
+      if (kRange) group = fmaxf(group, fabsf(x));
+      digits<kPlanes>(x, in && srl ? srl[c] * down : 0.f, d);
 #pragma unroll
       for (int t = 0; t < kPlanes; ++t) {
         if (j & 1) w[t][j / 2] |= d[t] & 0xffff0000u;
@@ -112,6 +138,18 @@ __global__ void __launch_bounds__(256) digit_rows_kernel(const float* __restrict
 #pragma unroll
     for (int t = 0; t < kPlanes; ++t)
       *reinterpret_cast<uint4*>(o + (size_t)t * tile * 128u) = make_uint4(w[t][0], w[t][1], w[t][2], w[t][3]);
+    if (kRange) {   // four adjacent lanes hold a group (their pieces exist or end together)
+      static_assert(kWideSites == 32, "four pieces of eight columns");
+      const unsigned quad = 0xfu << (threadIdx.x & 28);
+      group = fmaxf(group, __shfl_xor_sync(quad, group, 1));
+      group = fmaxf(group, __shfl_xor_sync(quad, group, 2));
+      below |= p / 4 * kWideSites + kWideSites <= n && group * kWideRatio < top;
+    }
+  }
+  if (kRange) below = __syncthreads_or(below);
+  if (threadIdx.x == 0) {
+    const float a = __uint_as_float(mx), f = finite ? __uint_as_float((uint32_t)(127 + e) << 23) : __uint_as_float(0x7fc00000u);
+    scale[r] = kRange && finite && (below || (mx > 0 && (a < 0x1p-100f || a >= 0x1p100f))) ? -f : f;
   }
 }
 
@@ -130,17 +168,43 @@ struct XArgs {
   const float* bscale;
   float2* part;          // kparts x R x n pairs
   int n, R, npad, nchunks, nblocks, kparts, cpp, items, ring;
+  const float *e, *hi, *lo;   // for the wide rows (CHAIN > 0): E (R x n) and the pair
+  int ld;
   uint32_t epi_wait;     // bound on the epilogue's waits for an accumulator (try_wait rounds)
   int* status;
 };
 
-__global__ void __launch_bounds__(kThreads) xprod_kernel(const __grid_constant__ XArgs p) {
+// The wide rows' FP32 products, after the digits: groups of 128 threads, each with its own part
+// of the block's shared memory (which no copy or product uses any more) and its own barrier.
+// Bound by the FP32 pipe at 12 warps per SM: n = 4500, R = 100, every row wide 582 us in all (the
+// FP32 form's own kernel, 20 warps per SM, 409); one wide row 209; none 80, as without this.
+template <int CHAIN>
+__device__ __forceinline__ void wide_rows(const XArgs& p, float* sm) {
+  constexpr int kGroups = xprod_threads(CHAIN) / 128;
+  static_assert(kGroups * SV_SMEM <= kMaxRing * kAPlane, "the smallest block (a full ring) holds the groups' tiles");
+  const int group = threadIdx.x >> 7, lane = threadIdx.x & 31;
+  const int ct = (p.n + SV_TC - 1) / SV_TC, per = ct * SV_KSPLIT;   // tiles of one block of rows
+  const int tiles = per * ((p.R + SV_TR - 1) / SV_TR);
+  for (int t = kGroups * blockIdx.x + group; t < tiles; t += kGroups * gridDim.x) {
+    const int r0 = t / per * SV_TR, c = t % per;
+    const uint32_t rows = __ballot_sync(0xffffffffu, r0 + lane < p.R && p.bscale[r0 + lane] < 0.f);
+    if (rows == 0) continue;
+    solve_tile<CHAIN>(p.e, p.R, p.n, p.hi, p.lo, p.ld, reinterpret_cast<float*>(p.part), c % ct * SV_TC, r0, c / ct, rows,
+                      threadIdx.x & 127, sm + group * (SV_SMEM / sizeof(float)),
+                      [&] { asm volatile("bar.sync %0, 128;" ::"r"(1 + group) : "memory"); });
+  }
+}
+
+// CHAIN: 0, or for the wide rows the FP32 product with that many terms per compensated step.
+template <int CHAIN>
+__global__ void __launch_bounds__(xprod_threads(CHAIN), 1) xprod_kernel(const __grid_constant__ XArgs p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   __shared__ __align__(8) uint64_t a_full[kMaxRing], a_empty[kMaxRing], b_full[2], b_empty[2], acc_full, acc_empty, drained;
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int any_wide = 0;
   const uint32_t bplane = (uint32_t)p.npad * 128u, bbuf = kBPlanes * bplane;
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.ring; ++s) {
@@ -296,7 +360,7 @@ __global__ void __launch_bounds__(kThreads) xprod_kernel(const __grid_constant__
       }
     }
     __syncwarp();
-  } else {
+  } else if (warp < kEpi) {
     // ------------------------------------------------------------ epilogue
     // thread: one row of the matrix tile, half of E's rows (columns of the accumulators)
     const int q = warp & 3, half = warp >> 2;
@@ -352,21 +416,33 @@ __global__ void __launch_bounds__(kThreads) xprod_kernel(const __grid_constant__
         float2* __restrict__ dst = p.part + (size_t)kp * p.R * p.n + i;
         const int rb = nb * p.npad + half * ncol;
 #pragma unroll
-        for (int j = 0; j < 64; ++j) {
-          if (j < ncol && rb + j < p.R) {
-            const float sc = p.bscale[rb + j];
-            float h = hi[j];   // a normalised pair: the low part is below half an ulp of the value
-            const float l = two_sum(h, lo[j]);
-            dst[(size_t)(rb + j) * p.n] = make_float2(h * as * sc, l * as * sc);
+        for (int g = 0; g < 8; ++g) {
+          float sc[8];   // negative: a wide row, whose pairs the FP32 products write
+#pragma unroll
+          for (int j = 0; j < 8; ++j) sc[j] = 8 * g + j < ncol ? p.bscale[rb + 8 * g + j] : 0.f;
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const int row = rb + 8 * g + j;
+            float h = hi[8 * g + j];   // a normalised pair: the low part is below half an ulp of the value
+            const float l = two_sum(h, lo[8 * g + j]);
+            const float f = CHAIN ? sc[j] : fabsf(sc[j]);
+            if (8 * g + j < ncol && row < p.R && !(f < 0.f)) dst[(size_t)row * p.n] = make_float2(h * as * f, l * as * f);
           }
         }
       }
     }
+  } else {
+    // ------------------------------------------------------------ are there wide rows (CHAIN > 0)
+    for (int r = threadIdx.x - (kEpi + 2) * 32; r < p.R; r += 64) any_wide |= p.bscale[r] < 0.f;
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   if (warp == kEpi) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+  if constexpr (CHAIN > 0) {
+    if (__syncthreads_or(any_wide) && !abort_flag)
+      wide_rows<CHAIN>(p, reinterpret_cast<float*>(smem_raw + (base - smem_u32(smem_raw))));
+  }
 }
 
 int nchunks_of(int n) { return (n + 63) / 64; }
@@ -398,8 +474,8 @@ size_t xprod_rows_bytes(int n, int R) {
   return (size_t)nb * nchunks_of(n) * kBPlanes * np * 128u + sizeof(float) * (size_t)nb * np;
 }
 
-int launch_xprod(ce_ctx* ctx, const float* E, long long lde, int R, int n, const void* matrix, void* rows,
-                 float* part, int max_parts, int* kparts_out, cudaStream_t s) {
+int launch_xprod(ce_ctx* ctx, const float* E, long long lde, int R, int n, const void* matrix, const XprodPair* pair,
+                 void* rows, float* part, int max_parts, int* kparts_out, const float** scale_out, cudaStream_t s) {
   const int np = block_rows(R), nb = (R + np - 1) / np, nc = nchunks_of(n), mt = mtiles_of(n);
   XArgs a;
   a.a = static_cast<const uint8_t*>(matrix);
@@ -414,6 +490,10 @@ int launch_xprod(ce_ctx* ctx, const float* E, long long lde, int R, int n, const
   a.npad = np;
   a.nchunks = nc;
   a.nblocks = nb;
+  a.e = E;
+  a.hi = pair ? pair->hi : nullptr;
+  a.lo = pair ? pair->lo : nullptr;
+  a.ld = pair ? pair->ld : 0;
   a.epi_wait = ctx->wait_limit;
   a.status = ctx->dev_status;
   int nsm = 0, dev = 0;
@@ -437,11 +517,13 @@ int launch_xprod(ce_ctx* ctx, const float* E, long long lde, int R, int n, const
   const uint32_t bbytes = 2u * kBPlanes * (uint32_t)np * 128u;
   a.ring = std::min<int>(kMaxRing, (int)((kXprodSmem - 1024u - bbytes) / kAPlane));
   const size_t smem = (size_t)bbytes + (size_t)a.ring * kAPlane + 1024;
-  CE_CUDA_TRY(set_max_smem(xprod_kernel, kXprodSmem));
+  auto kernel = !pair ? xprod_kernel<0> : (pair->chain == 2 ? xprod_kernel<2> : xprod_kernel<4>);
+  CE_CUDA_TRY(set_max_smem(kernel, kXprodSmem));
   digit_rows_kernel<kBPlanes><<<nb * np, 256, 0, s>>>(E, nullptr, lde, R, n, np, nc, planes, bscale);
-  xprod_kernel<<<std::min(a.items, nsm), kThreads, smem, s>>>(a);
+  kernel<<<std::min(a.items, nsm), xprod_threads(pair ? pair->chain : 0), smem, s>>>(a);
   CE_CUDA_TRY(cudaGetLastError());
   *kparts_out = kp;
+  if (scale_out) *scale_out = bscale;
   return CE_OK;
 }
 
