@@ -159,10 +159,10 @@ int ce_set_precision(ce_ctx* ctx, int prec);
 /* Form of the solve B = A^-1 E (Eq. (condmvn)) in ce_condsim, ce_solve and the batch
  * calls (no counterpart in the paper).  CE_SOLVE_FP32 (default): FP32 accuracy; from 1800
  * rows on the hi + lo pair of the FP64 inverse and E are cut into exact 8-bit digits whose
- * products the tensor cores sum (10 n_obs^2 bytes more device memory); below that, and for a
- * realization whose residuals lie below 1/128 of its largest one over a whole neighbourhood of
- * sites, FP32 products summed with error-free transformations.  B is within about 1e-7 of the
- * FP64 solve, in every part of the domain.  CE_SOLVE_TENSOR: tcgen05 tensor cores, A^-1 and E each
+ * products the tensor cores sum (10 n_obs^2 bytes more device memory); below that, where the
+ * set-up finds no room for the digits, and for a realization whose residuals lie below 1/128
+ * of its largest one over a whole neighbourhood of sites, FP32 products summed with error-free
+ * transformations.  B is within about 1e-7 of the FP64 solve, in every part of the domain.  CE_SOLVE_TENSOR: tcgen05 tensor cores, A^-1 and E each
  * split into f16 hi + lo (power-of-two scaled), three products, FP32 accumulation drained
  * every 512 sites, K split over work items whose partial products are joined in a fixed
  * order (deterministic); B is within about 1e-6 of the FP64 solve, at a fraction of the

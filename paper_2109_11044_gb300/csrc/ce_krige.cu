@@ -450,8 +450,10 @@ void launch_spd_cov(const GridC& g, const double* xy, int n, double diag_add, co
 }
 
 // The inverse of the prediction matrix in A (lower triangle, padded to nobs_pad) as the
-// context's FP32 pair.
-int store_inverse(ce_ctx* ctx, double* A, cudaStream_t s) {
+// context's FP32 pair, from kXprodMin rows on also as digits.  Frees A before it allocates the
+// digits (18 n^2 bytes at most in all, 16 while A lives); where there is no room for them, the
+// solve takes the FP32 products as it does for fewer rows.
+int store_inverse(ce_ctx* ctx, double*& A, cudaStream_t s) {
   const int n = ctx->nobs, ld = ctx->nobs_pad;
   int st = spd_inverse_f64(ctx, A, n, s, &ctx->logdet);
   if (st) return st;
@@ -464,13 +466,14 @@ int store_inverse(ce_ctx* ctx, double* A, cudaStream_t s) {
     CE_CUDA_TRY(cudaMemsetAsync(ctx->Ainv_lo, 0, bytes, s));
   }
   launch_finish_inverse(A, n, ctx->Ainv_hi, ctx->Ainv_lo, ld, s);
-  if (n >= kXprodMin) {
-    ctx->ainv_dig = dalloc(ctx, xprod_matrix_bytes(n));
-    if (!ctx->ainv_dig) return fail(ctx, CE_ERR_OOM, "digits of the inverse");
-    launch_xprod_matrix(ctx->Ainv_hi, ctx->Ainv_lo, ld, n, ctx->ainv_dig, s);
-  }
   CE_CUDA_TRY(cudaGetLastError());
   CE_CUDA_TRY(cudaStreamSynchronize(s));
+  dfree(ctx, A);
+  A = nullptr;
+  if (n >= kXprodMin && (ctx->ainv_dig = dalloc(ctx, xprod_matrix_bytes(n)))) {
+    launch_xprod_matrix(ctx->Ainv_hi, ctx->Ainv_lo, ld, n, ctx->ainv_dig, s);   // (the caller synchronises)
+    CE_CUDA_TRY(cudaGetLastError());
+  }
   return CE_OK;
 }
 
