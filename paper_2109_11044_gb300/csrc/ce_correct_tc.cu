@@ -359,19 +359,16 @@ __global__ void __maxnreg__(TcRoles<NPW>::MAXREG) correct_tc_kernel(const __grid
       if (item.x < 0) break;
       const TcEvent& ev = p.ev[MULTI ? item.x : 0];   // one event: fixed parameter offsets
       const float absb = ev.absb, c1 = ev.c1;
-      // Offsets are formed from the row's multiple of four, then shifted by the row's
-      // remainder of nodes along x (anisotropic: by the shift's image under the map, whose
-      // first column is (a11, a21)).  Values travel in pairs of adjacent sites.
-      const float rem = (float)(base_row & 3);
-      const float ubf = ANISO ? rem * absb * p.a11 : rem * absb, vbf = ANISO ? rem * absb * p.a21 : 0.f;
-      const uint64_t ub = pack2(ubf, ubf), vb = pack2(vbf, vbf), absb2 = pack2(absb, absb);
+      // Offsets are formed from each row's own node (one rounding each).  Values travel in pairs of
+      // adjacent sites.
+      const uint64_t absb2 = pack2(absb, absb);
       const uint64_t tiny2 = pack2(1e-30f, 1e-30f), scale2 = pack2(kLoScale, kLoScale), c1n = pack2(-c1, -c1);
       // the event's fields in registers (a parameter-space read per use would be slow)
       const int nchunks = ev.nchunks;
       const ulonglong2* __restrict__ sites = reinterpret_cast<const ulonglong2*>(ev.sites) + c * SPC;
       const int tpr = ev.tiles_per_row;
       const float fgi = (float)(item.y / tpr);
-      const float fgj0 = (float)((item.y % tpr) * TM + (base_row & ~3));
+      const float fgj0 = (float)((item.y % tpr) * TM + base_row);
       const uint64_t fgi2 = pack2(fgi, fgi);
       for (int kc = 0; kc < nchunks; ++kc, stage_ring.next(), gsel = gsel + 1 == Ro::NGROUP ? 0 : gsel + 1) {
         if (gsel != grp) continue;
@@ -408,12 +405,11 @@ __global__ void __maxnreg__(TcRoles<NPW>::MAXREG) correct_tc_kernel(const __grid
               uint64_t d2;
               if (ANISO) {
                 const float2 xy0 = unpack2(dx), xy1 = unpack2(dy[j]);
-                const uint64_t du = add2(pack2(fmaf(p.a11, xy0.x, p.a12 * xy1.x), fmaf(p.a11, xy0.y, p.a12 * xy1.y)), ub);
-                const uint64_t dv = add2(pack2(fmaf(p.a21, xy0.x, p.a22 * xy1.x), fmaf(p.a21, xy0.y, p.a22 * xy1.y)), vb);
+                const uint64_t du = pack2(fmaf(p.a11, xy0.x, p.a12 * xy1.x), fmaf(p.a11, xy0.y, p.a12 * xy1.y));
+                const uint64_t dv = pack2(fmaf(p.a21, xy0.x, p.a22 * xy1.x), fmaf(p.a21, xy0.y, p.a22 * xy1.y));
                 d2 = fma2(du, du, fma2(dv, dv, tiny2));
               } else {
-                const uint64_t du = add2(dx, ub);
-                d2 = fma2(du, du, dy[j]);
+                d2 = fma2(dx, dx, dy[j]);
               }
               // |b| d (distances are in units of the exponent scale) and 2^-|b| d
               const float2 q = unpack2(d2);
