@@ -252,8 +252,8 @@ int ce_set_box_joint(ce_ctx* ctx, int on, int* n_boxes);
  * M x n by n x n (M grid nodes; 177 ms in all at 512 x 512, n = 2000, 36 window
  * nodes).  Allocates its work buffers (about 300 MB
  * at most; se_approx in local mode: 18 n^2 bytes more for Q's pair and digits, and an
- * m x (2m - 1) table), synchronises `stream` and returns a status that a kernel
- * recorded, as ce_condsim_host does. */
+ * m x (2m - 1) table), synchronises `stream` and, for se_approx in local mode, returns a
+ * status that a kernel recorded, as ce_condsim_host does. */
 int ce_se_map(ce_ctx* ctx, float* se_exact_dev, float* se_approx_dev, void* stream);
 
 /* Ensemble moments at every grid node (the ensemble mean estimate and its

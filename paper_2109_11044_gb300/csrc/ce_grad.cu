@@ -365,10 +365,13 @@ __global__ void window_sumsq_kernel(const float* __restrict__ v, int m, Window w
   if (threadIdx.x == 0) atomicAdd(acc, t);
 }
 
-// dL/dz[caller index perm[q]] = sum_r w_r,q - alpha_q.
+// dL/dz[caller index perm[q]] = sum_r w_r,q - alpha_q; *out_status = *status (the call's kernels
+// before this one have recorded theirs).
 __global__ void grad_z_kernel(const float* __restrict__ w, const float* __restrict__ alpha, int R, int nobs,
-                              const int* __restrict__ perm, float* __restrict__ gz) {
+                              const int* __restrict__ perm, float* __restrict__ gz, const int* __restrict__ status,
+                              double* __restrict__ out_status) {
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q == 0) *out_status = (double)*status;
   if (q >= nobs) return;
   float s = 0.f;
   for (int r = 0; r < R; ++r) s += w[(long long)r * nobs + q];
@@ -458,7 +461,9 @@ extern "C" int ce_condsim_grad(ce_ctx* ctx, const float* z_dev, int R, uint64_t 
         csum, dsum, ctx->Bm, ctx->nobs_pad, R, n, f, inv_sigma, c, acc + 0);
   }
   // 2. w = A^-1 c
-  if ((st = launch_solve(ctx, c, R, w, n, s, nullptr))) { dfree(ctx, acc); return st; }
+  // c decays away from the window.  w enters sums with alpha and over all sites, so an error relative to
+  // a row's largest value (2^-33 by the digits) is below their rounding (2^-25): no row counts as wide
+  if ((st = launch_solve(ctx, c, R, w, n, s, nullptr, false))) { dfree(ctx, acc); return st; }
   // 3. prediction matrix and log-likelihood
   {
     const size_t shm = sizeof(float) * 2 * (size_t)R * GP_T;
@@ -476,7 +481,7 @@ extern "C" int ce_condsim_grad(ce_ctx* ctx, const float* z_dev, int R, uint64_t 
   // 5. the unconditional fields, through the spectral weights
   if ((st = launch_adjoint_ensemble(ctx, H, R, seed, r_offset, acc + 8, s))) { dfree(ctx, acc); return st; }
   // 6. dL/dz, loss
-  grad_z_kernel<<<(n + 255) / 256, 256, 0, s>>>(w, alpha, R, n, ctx->perm, grad_z_dev);
+  grad_z_kernel<<<(n + 255) / 256, 256, 0, s>>>(w, alpha, R, n, ctx->perm, grad_z_dev, ctx->dev_status, acc + 11);
   window_sumsq_kernel<<<256, 256, 0, s>>>(out_dev, ctx->m, win, R, acc + 10);
   CE_CUDA_TRY(cudaGetLastError());
   double h_acc[16];
@@ -485,11 +490,11 @@ extern "C" int ce_condsim_grad(ce_ctx* ctx, const float* z_dev, int R, uint64_t 
   CE_CUDA_TRY(cudaMemcpyAsync(h_acc, acc, sizeof(h_acc), cudaMemcpyDeviceToHost, s));
   CE_CUDA_TRY(cudaMemcpyAsync(h_alpha.data(), alpha, sizeof(float) * n, cudaMemcpyDeviceToHost, s));
   CE_CUDA_TRY(cudaMemcpyAsync(h_z.data(), ctx->zint, sizeof(float) * n, cudaMemcpyDeviceToHost, s));
-  st = sync_stream_status(ctx, s);   // an expired wait left incomplete sums
+  CE_CUDA_TRY(cudaStreamSynchronize(s));
   dfree(ctx, acc);
-  if (st) return st;
+  if (h_acc[11] != 0.0 && (st = sync_stream_status(ctx, s))) return st;   // an expired wait left incomplete sums
   // acc: [0,1] correction (sigma, theta); [2,3,4] pairs (sigma, theta, tau2);
-  //      [5,6,7] off-grid (sigma, theta, tau2); [8,9] fields (theta, sigma); [10] sum of squares
+  //      [5,6,7] off-grid (sigma, theta, tau2); [8,9] fields (theta, sigma); [10] sum of squares; [11] status
   grad_theta[0] = h_acc[0] + h_acc[2] + h_acc[5] + h_acc[9];
   grad_theta[1] = h_acc[1] + h_acc[3] + h_acc[6] + h_acc[8];
   grad_theta[2] = h_acc[4] + h_acc[7];

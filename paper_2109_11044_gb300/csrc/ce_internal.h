@@ -169,8 +169,9 @@ void launch_finish_inverse(double* M, int n, float* hi, float* lo, int ld, cudaS
 void gemm64_nn_sub(const double* A, int lda, const double* B, int ldb, double* C, int ldc, int M, int N, int K,
                    cudaStream_t s);
 // B = A^-1 E with the stored pair, through the context's Bpart (and xrows); *launches counts
-// its kernels (may be null).
-int launch_solve(ce_ctx* ctx, const float* E, int R, float* B, int ldb, cudaStream_t s, int* launches);
+// its kernels (may be null).  wide_rows: rows of wide range keep their accuracy at every site
+// (XprodPair), not only relative to their largest value.
+int launch_solve(ce_ctx* ctx, const float* E, int R, float* B, int ldb, cudaStream_t s, int* launches, bool wide_rows = true);
 // ce_xprod.cu: E A^-1 on the tensor cores from 8-bit digits.  The digit planes of the n x n
 // pair hi + lo (row stride ld), in a buffer of xprod_matrix_bytes(n); those of R rows of E
 // take xprod_rows_bytes(n, R).  launch_xprod writes *kparts <= max_parts partial (sum,

@@ -61,8 +61,9 @@ __global__ void __launch_bounds__(128, CHAIN == 4 ? 4 : 5) solve_gemm_f32(const 
 // float pair (TwoSum of the sums, the compensations and the TwoSum errors gathered in
 // a second float: FP64 arithmetic is slow on this part), rounded once.  PARTS: their number
 // where it is fixed, so that all loads are in flight (1500 rows, R = 60, the whole solve: 45.5 us
-// with a runtime count, 43.5 with this one); 0 takes `parts`, or SV_KSPLIT where scale[r] < 0.
-template <int PARTS>
+// with a runtime count, 43.5 with this one); 0 takes `parts`, or (WIDE) SV_KSPLIT where
+// scale[r] < 0.
+template <int PARTS, bool WIDE>
 __global__ void solve_reduce(const float* __restrict__ part, int parts, const float* __restrict__ scale, int R, int n,
                              float* __restrict__ Bout, int ldb) {
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -82,7 +83,7 @@ __global__ void solve_reduce(const float* __restrict__ part, int parts, const fl
 #pragma unroll
     for (int k = 0; k < PARTS; ++k) add(k);
   } else {
-    const bool w = scale[r] < 0.f;   // read beside the first pairs, which every row has
+    const bool w = WIDE && scale[r] < 0.f;   // read beside the first pairs, which every row has
 #pragma unroll 4
     for (int k = 0; k < parts; ++k) add(k);
     if (w)
@@ -121,7 +122,7 @@ void gemm64_nn_sub(const double* A, int lda, const double* B, int ldb, double* C
   gemm64_sub<<<g, 256, 0, s>>>(A, lda, B, ldb, C, ldc, M, N, K);
 }
 
-int launch_solve(ce_ctx* ctx, const float* E, int R, float* B, int ldb, cudaStream_t s, int* launches) {
+int launch_solve(ce_ctx* ctx, const float* E, int R, float* B, int ldb, cudaStream_t s, int* launches, bool wide_rows) {
   const int n = ctx->nobs, ld = ctx->nobs_pad;
   const unsigned rb = (unsigned)(((long long)R * n + 255) / 256);
   // the FP32 form's products in pairs (the tightest error); the tensor forms, whose correction
@@ -131,16 +132,17 @@ int launch_solve(ce_ctx* ctx, const float* E, int R, float* B, int ldb, cudaStre
     int parts = 0;
     const float* scale = nullptr;   // negative: SV_KSPLIT partial pairs
     const XprodPair pair{ctx->Ainv_hi, ctx->Ainv_lo, ld, pairs ? 2 : 4};
-    const int st = launch_xprod(ctx, E, n, R, n, ctx->ainv_dig, &pair, ctx->xrows, ctx->Bpart, SV_KSPLIT, &parts, &scale, s);
+    const int st = launch_xprod(ctx, E, n, R, n, ctx->ainv_dig, wide_rows ? &pair : nullptr, ctx->xrows, ctx->Bpart, SV_KSPLIT, &parts, &scale, s);
     if (st) return st;
-    solve_reduce<0><<<rb, 256, 0, s>>>(ctx->Bpart, parts, scale, R, n, B, ldb);
+    auto reduce = wide_rows ? solve_reduce<0, true> : solve_reduce<0, false>;
+    reduce<<<rb, 256, 0, s>>>(ctx->Bpart, parts, scale, R, n, B, ldb);
     if (launches) *launches += 3;
     return CE_OK;
   }
   auto gemm = pairs ? solve_gemm_f32<2> : solve_gemm_f32<4>;
   gemm<<<dim3((n + SV_TC - 1) / SV_TC, (R + SV_TR - 1) / SV_TR, SV_KSPLIT), 128, 0, s>>>(E, R, n, ctx->Ainv_hi, ctx->Ainv_lo, ld,
                                                                                       ctx->Bpart);
-  solve_reduce<SV_KSPLIT><<<rb, 256, 0, s>>>(ctx->Bpart, SV_KSPLIT, nullptr, R, n, B, ldb);
+  solve_reduce<SV_KSPLIT, false><<<rb, 256, 0, s>>>(ctx->Bpart, SV_KSPLIT, nullptr, R, n, B, ldb);
   if (launches) *launches += 2;
   return CE_OK;
 }

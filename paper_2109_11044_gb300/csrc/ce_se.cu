@@ -535,9 +535,11 @@ extern "C" int ce_se_map(ce_ctx* ctx, float* se_exact_dev, float* se_approx_dev,
     }
   }
   cudaError_t e = cudaGetLastError();
-  const int dev = sync_stream_status(ctx, s);   // an expired wait left an incomplete product
+  const cudaError_t e2 = cudaStreamSynchronize(s);
   release();
   if (st) return st;
+  if (e == cudaSuccess) e = e2;
   if (e != cudaSuccess) return cuda_fail(e, "standard errors", __FILE__, __LINE__);
-  return dev;
+  // the digit product's waits are bounded: one that expired has left an incomplete product
+  return need_u ? sync_stream_status(ctx, s) : CE_OK;
 }

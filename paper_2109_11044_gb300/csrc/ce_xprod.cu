@@ -85,12 +85,11 @@ constexpr float kWideRatio = 128.f;
 // null), one block per row.  Row r goes to row r % tile of tile r / tile: planes of tile x
 // 128 bytes, kPlanes of them per chunk of 64 columns, nchunks chunks per tile.  Rows past
 // `rows` and columns past n are zeros.  scale[r]: the power of two to multiply back by
-// (NaN where the row is not finite), negative for a wide row of E.
-template <int kPlanes>
+// (NaN where the row is not finite), with kRange negative for a wide row.
+template <int kPlanes, bool kRange>
 __global__ void __launch_bounds__(256) digit_rows_kernel(const float* __restrict__ v, const float* __restrict__ lo, long long ldv,
                                                          int rows, int n, int tile, int nchunks, uint8_t* __restrict__ out,
                                                          float* __restrict__ scale) {
-  constexpr bool kRange = kPlanes == kBPlanes;
   __shared__ unsigned wmax[8];
   const int r = blockIdx.x;
   const bool live = r < rows;
@@ -425,8 +424,7 @@ __global__ void __launch_bounds__(xprod_threads(CHAIN), 1) xprod_kernel(const __
             const int row = rb + 8 * g + j;
             float h = hi[8 * g + j];   // a normalised pair: the low part is below half an ulp of the value
             const float l = two_sum(h, lo[8 * g + j]);
-            const float f = CHAIN ? sc[j] : fabsf(sc[j]);
-            if (8 * g + j < ncol && row < p.R && !(f < 0.f)) dst[(size_t)row * p.n] = make_float2(h * as * f, l * as * f);
+            if (8 * g + j < ncol && row < p.R && !(sc[j] < 0.f)) dst[(size_t)row * p.n] = make_float2(h * as * sc[j], l * as * sc[j]);
           }
         }
       }
@@ -458,7 +456,7 @@ void launch_xprod_matrix(const float* hi, const float* lo, int ld, int n, void* 
   const int mt = mtiles_of(n), nc = nchunks_of(n);
   uint8_t* planes = static_cast<uint8_t*>(buf);
   float* scale = reinterpret_cast<float*>(planes + (size_t)mt * nc * kAPlanes * kAPlane);
-  digit_rows_kernel<kAPlanes><<<mt * 128, 256, 0, s>>>(hi, lo, ld, n, n, 128, nc, planes, scale);
+  digit_rows_kernel<kAPlanes, false><<<mt * 128, 256, 0, s>>>(hi, lo, ld, n, n, 128, nc, planes, scale);
 }
 
 namespace {
@@ -519,7 +517,8 @@ int launch_xprod(ce_ctx* ctx, const float* E, long long lde, int R, int n, const
   const size_t smem = (size_t)bbytes + (size_t)a.ring * kAPlane + 1024;
   auto kernel = !pair ? xprod_kernel<0> : (pair->chain == 2 ? xprod_kernel<2> : xprod_kernel<4>);
   CE_CUDA_TRY(set_max_smem(kernel, kXprodSmem));
-  digit_rows_kernel<kBPlanes><<<nb * np, 256, 0, s>>>(E, nullptr, lde, R, n, np, nc, planes, bscale);
+  auto rows_kernel = pair ? digit_rows_kernel<kBPlanes, true> : digit_rows_kernel<kBPlanes, false>;
+  rows_kernel<<<nb * np, 256, 0, s>>>(E, nullptr, lde, R, n, np, nc, planes, bscale);
   kernel<<<std::min(a.items, nsm), xprod_threads(pair ? pair->chain : 0), smem, s>>>(a);
   CE_CUDA_TRY(cudaGetLastError());
   *kparts_out = kp;
