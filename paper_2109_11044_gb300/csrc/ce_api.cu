@@ -1,6 +1,5 @@
 // C ABI of the library: argument checks, context and buffer management, and
 // the order of the steps of the conditional simulation (Section 2, steps 1-5).
-#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -74,11 +73,7 @@ int ensure_work(ce_ctx* ctx, int R) {
   ctx->E = (float*)dalloc(ctx, sizeof(float) * (size_t)R * ctx->nobs);
   ctx->Bm = (float*)dalloc(ctx, sizeof(float) * (size_t)Rpad * ctx->nobs_pad);
   ctx->Bpart = (float*)dalloc(ctx, sizeof(float2) * kSolveKSplit * (size_t)R * ctx->nobs);   // (sum, compensation) pairs
-  if (ctx->ainv_dig) {
-    size_t rows = 0;   // the padding of the blocks of rows is not monotone in R
-    for (int r = 1; r <= R; ++r) rows = std::max(rows, xprod_rows_bytes(ctx->nobs, r));
-    ctx->xrows = dalloc(ctx, rows);
-  }
+  if (ctx->ainv_dig) ctx->xrows = dalloc(ctx, xprod_rows_bytes(ctx->nobs, R));   // enough for fewer rows too
   if (!ctx->E || !ctx->Bm || !ctx->Bpart || (ctx->ainv_dig && !ctx->xrows)) return fail(ctx, CE_ERR_OOM, "per-call buffers");
   CE_CUDA_TRY(cudaMemset(ctx->Bm, 0, sizeof(float) * (size_t)Rpad * ctx->nobs_pad));
   ctx->Rcap = R;
