@@ -154,9 +154,9 @@ __device__ __forceinline__ uint32_t pack_f16x2(float lo_elem, float hi_elem) {
 // Two FP32 values in one 64-bit register pair, for the packed add, multiply and FMA
 // (each half rounded as the scalar instruction rounds it).  The producers are bound by
 // instruction issue and latency, not by a pipe; one packed instruction for two adjacent
-// sites takes the kernel from 260 M to 221 M warp instructions at 512 x 512 nodes, 2000
-// sites, R = 100 (0.367 -> 0.342 ms) and 10.5 -> 9.9 ms at 2048 x 2048, 4000 sites,
-// R = 32, with the same bits.
+// sites took the kernel from 260 M to 221 M warp instructions at 512 x 512 nodes, 2000
+// sites, R = 100 (367 -> 342 us; 218 M and 330 us now), and from 10.5 to 9.9 ms at 2048 x
+// 2048, 4000 sites, R = 32 (8.15 ms now).
 __device__ __forceinline__ uint64_t pack2(float x, float y) {
   uint64_t d;
   asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));

@@ -22,7 +22,9 @@
 // operands' way through L2 (10 bytes per matrix element).  n = 4500, R = 100: 0.385 ms (the
 // FP32 form) -> 0.053 ms; n = 2000, R = 100: 84 -> 17 us.  Below n = 1800 (kXprodMin) its
 // fixed cost (digits, launch, tensor-memory set-up: 11 us for any small n) exceeds the FP32
-// form's time at small R (n = 1000: 13 us at R = 8 against 8); at 2000 they meet at R = 1.
+// form's time at small R (n = 1000: 13 us at R = 8 against 8).  The whole solve in FP32 and in
+// digits: n = 1800, R = 1: 30.1 and 30.0 us, R = 4: 29.0 and 33.1; n = 1900, R = 16: 35.3 and
+// 33.2; n = 2000, R = 8: 32.8 and 33.9, R = 100: 100 and 38; n = 2500, R = 1: 38.4 and 38.4.
 // The line is drawn by n alone, never by R: a realization's result must not depend on how
 // many others are solved with it.
 // One block per SM: a loader lane (bulk copies of the matrix's digit planes into a ring, of
